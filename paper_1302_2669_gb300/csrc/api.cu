@@ -179,6 +179,12 @@ int widen_lanes(const surfmcmc_ctx* ctx, int L, int requested, int lam, long lon
     return widen_lanes_for(ctx->sms, L, lam, n_bundles, G, code);
 }
 
+// Whether a planned run takes the one-block-per-bundle kernel (wide_batch):
+// not when the caller fixed the lanes.
+int take_wide(const surfmcmc_ctx* ctx, const surfmcmc_opts& o, const SweepParams& sp) {
+    return o.lanes_per_bundle ? 0 : wide_batch(ctx->sms, sp);
+}
+
 int check_opts(surfmcmc_ctx* ctx, const surfmcmc_opts& o, double p) {
     if (o.noise < 0 || o.noise > 2) return fail(ctx, SURFMCMC_EINVAL, "noise=%d must be 0, 1 or 2", o.noise);
     if (o.noise != 1 && !(p > 0.0 && p <= 0.75)) return fail(ctx, SURFMCMC_EINVAL, "p=%g outside (0, 0.75]", p);
@@ -408,6 +414,7 @@ int ragged_layout(surfmcmc_ctx* ctx, const int32_t* Ls, const uint32_t* sweeps, 
     }
     lay.e0_words = e0w;
     lay.state_words = stw;
+    lay.sp.wide = take_wide(ctx, o, lay.sp);
     return SURFMCMC_OK;
 }
 
@@ -827,6 +834,7 @@ int surfmcmc_decode_ex(surfmcmc_ctx* ctx, const uint8_t* syndromes, int64_t n, i
     if (!init_frames) CK(launch_start_frames((const uint8_t*)b_syn.dev, n, L, e0, code, s, toric));
     if (accepts) CK(cudaMemsetAsync(accepts, 0, (size_t)n * Cn * 8, s));
     sp.accepts = accepts;   // every launch adds to the counts
+    sp.wide = take_wide(ctx, o, sp);
 
     SweepIO io;
     io.e0 = e0;
@@ -911,6 +919,7 @@ int surfmcmc_decode_ti(surfmcmc_ctx* ctx, const uint8_t* syndromes, int64_t n, i
     // results do not depend on the lane split)
     lam = widen_lanes(ctx, L, o.lanes_per_bundle, lam, bundles_of(sp, n), sp.G, toric);
     add_group(sp, L, n, 0, 0, 0, 0, lam);
+    sp.wide = take_wide(ctx, o, sp);
     const std::vector<Segment> segs0 = plan_segments(o, o.beta_scale, 0);
     const int W = geo_words(toric, L), nq = geo_nq(toric, L);
 
@@ -1289,6 +1298,7 @@ int surfmcmc_decode_early(surfmcmc_ctx* ctx, surfmcmc_cnn* net, const uint8_t* s
         sp.ids = t == 0 ? nullptr : (const uint32_t*)at(off_ids[cur]);
         const int lam_k = widen_lanes(ctx, L, o.lanes_per_bundle, lam, bundles_of(sp, n_act), sp.G);
         add_group(sp, L, n_act, 0, 0, 0, 0, lam_k);
+        sp.wide = take_wide(ctx, o, sp);
         make_round_keys((uint32_t)seed, (uint32_t)(seed >> 32), &sp.rk);
         // the chunk's non-empty segments (annealing stages already passed are skipped)
         std::vector<Segment> segs;

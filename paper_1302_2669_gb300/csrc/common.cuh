@@ -228,6 +228,7 @@ struct SweepParams {
     // Threshold bits of plane k as the algebraic normal form of the map
     // d-1 = e0 + 2 e1 -> bit (31-k) of T[d]: f = c0 ^ e0 c1 ^ e1 c2 ^ e0 e1 c3.
     uint32_t pc[4][32];
+    uint32_t tb[4][32];        // the same bits as masks: bit (31-k) of T[d] at [d-1][k] (one-block-per-bundle kernel)
     const uint32_t* e0;        // pure errors
     const int32_t* e0code;     // [items]
     const uint32_t* init_frames;  // per-chain start frames, or NULL
@@ -243,6 +244,7 @@ struct SweepParams {
     long long total_units;
     unsigned int* unit_counter;   // work queue of the persistent blocks (reset by the launcher)
     int max_blocks_per_sm;        // persistent blocks per multiprocessor, at most (0: as many as fit)
+    int wide;                     // > 0: one block of at most so many threads per bundle (small batches, sweep_wide.cu)
     GroupDesc grp[kMaxGroups];
 };
 
@@ -265,6 +267,8 @@ cudaError_t launch_sweep_flips(const SweepParams& p, int lanes_per_bundle, cudaS
 // The launch on a kernel with its digit-plane modes compiled in;
 // cudaErrorNotSupported (nothing launched) where there is none.
 cudaError_t launch_sweep_modes(const SweepParams& p, int lanes_per_bundle, cudaStream_t s);
+// The launch with one block per bundle (colour sweeps without accept counts).
+cudaError_t launch_sweep_wide(const SweepParams& p, cudaStream_t s);
 cudaError_t prepare_sweep_flips(const SweepParams& p, int lanes_per_bundle);
 cudaError_t prepare_sweep(const SweepParams& p, int lanes_per_bundle);
 size_t sweep_smem_bytes(int nq, int nc, int lanes_per_bundle);  // dynamic shared memory of a block

@@ -111,6 +111,7 @@ extern "C" int surfmcmc_decode_noalloc(const uint8_t* syndromes, int64_t n, int3
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return SURFMCMC_ECUDA;
     const int lam = widen_lanes_for(sms, L, heuristic_lanes(L, 0), bundles_of(sp, n), sp.G, 0);
     add_group(sp, L, n, 0, 0, 0, 0, lam);
+    sp.wide = wide_batch(sms, sp);
     GroupDesc& gd = sp.grp[0];
     gd.t_begin = 0;
     gd.t_end = o.n_sweeps;

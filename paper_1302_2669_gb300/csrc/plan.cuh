@@ -95,6 +95,7 @@ inline void set_temperature(SweepParams& sp, double p, double beta_scale) {
         sp.pc[1][k] = (t[1] ^ t[2]) ? ~0u : 0u;
         sp.pc[2][k] = (t[1] ^ t[3]) ? ~0u : 0u;
         sp.pc[3][k] = (t[1] ^ t[2] ^ t[3] ^ t[4]) ? ~0u : 0u;
+        for (int d = 1; d <= 4; ++d) sp.tb[d - 1][k] = t[d] ? ~0u : 0u;
     }
 }
 
@@ -132,6 +133,21 @@ inline int widen_lanes_for(int sms, int L, int lam, long long n_bundles, int G, 
     while (lam < 32 && sweep_units(n_bundles, lam) < capacity && sweep_smem_bytes(nq, nc, 2 * lam) <= kSweepSmemLimit)
         lam *= 2;
     return lam;
+}
+
+// Thread budget of the one-block-per-bundle kernel (sweep_wide.cu) for a
+// launch; 0: the launch takes the throughput kernel.  Up to 4 bundles per
+// multiprocessor it is the faster one at every size measured (L = 5: 211
+// against 333 us for 60 sweeps, L = 25: 1618 against 1766); from 8 on it is
+// not.  The budget shares a multiprocessor's 1024 threads (64 registers
+// each) among its bundles.
+inline int wide_batch(int sms, const SweepParams& sp) {
+    if (sp.scan || sp.accepts || sms <= 0) return 0;
+    long long bundles = 0;
+    for (int g = 0; g < sp.n_groups; ++g) bundles += sp.grp[g].n_bundles;
+    if (bundles > 4LL * sms) return 0;
+    const long long per_sm = (bundles + sms - 1) / sms;
+    return (int)(1024 / (per_sm < 1 ? 1 : per_sm > 4 ? 4 : per_sm));
 }
 
 // Chain layout of a run: C chains per syndrome, plane width G, bundles of 32

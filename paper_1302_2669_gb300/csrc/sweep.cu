@@ -20,6 +20,7 @@ cudaError_t prepare_sweep(const SweepParams& p, int lam) {
 }
 
 cudaError_t launch_sweep(const SweepParams& p, int lam, cudaStream_t s) {
+    if (p.wide) return launch_sweep_wide(p, s);
     // kernels with the launch's digit-plane modes compiled in, where they exist
     const cudaError_t e = launch_sweep_modes(p, lam, s);
     if (e != cudaErrorNotSupported) return e;

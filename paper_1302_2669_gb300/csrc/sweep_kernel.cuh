@@ -233,42 +233,55 @@ struct PlaneBatch {
 
     __device__ __forceinline__ void make(const SweepParams& p, const uint32_t* sid, uint32_t w, uint32_t t,
                                          uint32_t colm, uint32_t bt) {
+        uint4 b[SLOTS];
+#pragma unroll
+        for (int s = 0; s < SLOTS; ++s)
+            b[s] = philox10(make_uint4(sid[s], t, colm, G == 32 ? (w << 8) | bt : bt), p.rk);
+        merge(b);
+    }
+
+    // The planes from the blocks of the bundle's SLOTS syndromes.
+    __device__ __forceinline__ void merge(const uint4 b[SLOTS]) {
         if constexpr (G == 32) {
-            const uint4 b = philox10(make_uint4(sid[0], t, colm, (w << 8) | bt), p.rk);
-            pl[0] = b.x; pl[1] = b.y; pl[2] = b.z; pl[3] = b.w;
+            pl[0] = b[0].x; pl[1] = b[0].y; pl[2] = b[0].z; pl[3] = b[0].w;
         } else if constexpr (G == 16) {
-            merge16(philox10(make_uint4(sid[0], t, colm, bt), p.rk), philox10(make_uint4(sid[1], t, colm, bt), p.rk));
-        } else if constexpr (G == 8) {
-            uint32_t bw[4][4];
+            merge16(b[0], b[1]);
+        } else {
+            uint32_t bw[SLOTS][4];
 #pragma unroll
-            for (int s = 0; s < 4; ++s) {
-                const uint4 b = philox10(make_uint4(sid[s], t, colm, bt), p.rk);
-                bw[s][0] = b.x; bw[s][1] = b.y; bw[s][2] = b.z; bw[s][3] = b.w;
+            for (int s = 0; s < SLOTS; ++s) {
+                bw[s][0] = b[s].x; bw[s][1] = b[s].y; bw[s][2] = b[s].z; bw[s][3] = b[s].w;
             }
 #pragma unroll
-            for (int k = 0; k < 16; ++k) {
-                const int wi = k / 4, by = k % 4;
-                const uint32_t sel = (uint32_t)(by | ((4 + by) << 4));
-                const uint32_t lo = __byte_perm(bw[0][wi], bw[1][wi], sel);
-                const uint32_t hi = __byte_perm(bw[2][wi], bw[3][wi], sel);
-                pl[k] = __byte_perm(lo, hi, 0x5410);
-            }
-        } else {  // G == 4
-            uint32_t bw[8][4];
+            for (int wi = 0; wi < 4; ++wi) {
+                if constexpr (G == 8) {
+                    transpose4(bw[0][wi], bw[1][wi], bw[2][wi], bw[3][wi], pl + 4 * wi, 1);
+                } else {
+                    // 8 x 8 nibbles: nibble pairs of two syndromes first, then
+                    // bytes (32 operations; one nibble at a time took 128)
+                    uint32_t lo[4], hi[4];
 #pragma unroll
-            for (int s = 0; s < 8; ++s) {
-                const uint4 b = philox10(make_uint4(sid[s], t, colm, bt), p.rk);
-                bw[s][0] = b.x; bw[s][1] = b.y; bw[s][2] = b.z; bw[s][3] = b.w;
-            }
-#pragma unroll
-            for (int k = 0; k < 32; ++k) {
-                const int wi = k / 8, sh = 4 * (k % 8);
-                uint32_t v = 0;
-#pragma unroll
-                for (int s = 0; s < 8; ++s) v |= ((bw[s][wi] >> sh) & 0xFu) << (4 * s);
-                pl[k] = v;
+                    for (int i = 0; i < 4; ++i) {
+                        const uint32_t x = bw[2 * i][wi], y = bw[2 * i + 1][wi];
+                        lo[i] = (x & 0x0F0F0F0Fu) | ((y << 4) & 0xF0F0F0F0u);
+                        hi[i] = ((x >> 4) & 0x0F0F0F0Fu) | (y & 0xF0F0F0F0u);
+                    }
+                    transpose4(lo[0], lo[1], lo[2], lo[3], pl + 8 * wi, 2);
+                    transpose4(hi[0], hi[1], hi[2], hi[3], pl + 8 * wi + 1, 2);
+                }
             }
         }
+    }
+
+    // Byte j of the four words, in order, as out[j step], j = 0..3.
+    __device__ __forceinline__ static void transpose4(uint32_t a, uint32_t b, uint32_t c, uint32_t d, uint32_t* out,
+                                                      int step) {
+        const uint32_t ab0 = __byte_perm(a, b, 0x5140), ab1 = __byte_perm(a, b, 0x7362);
+        const uint32_t cd0 = __byte_perm(c, d, 0x5140), cd1 = __byte_perm(c, d, 0x7362);
+        out[0] = __byte_perm(ab0, cd0, 0x5410);
+        out[step] = __byte_perm(ab0, cd0, 0x7632);
+        out[2 * step] = __byte_perm(ab1, cd1, 0x5410);
+        out[3 * step] = __byte_perm(ab1, cd1, 0x7632);
     }
 
     // The same planes for block bt of the head from the bundle's fixed
@@ -521,6 +534,116 @@ __device__ __forceinline__ void acpt_add(uint32_t* a, uint32_t acc, uint32_t val
     if (++a[32 * kAcptPlanes] == kAcptCapacity) acpt_flush(a, valid, accepts, ci_of);
 }
 
+// The syndromes and chains behind a bundle's 32 bits: bit b belongs to chain
+// chain_of(b) of the syndrome with global item index syn_of(b); bits outside
+// `valid` (a partly filled bundle) belong to no chain.
+template <int G>
+struct BundleMap {
+    static constexpr int SLOTS = PlaneBatch<G>::SLOTS;
+    long long syn[SLOTS];
+    uint32_t sid[SLOTS];
+    uint32_t w, valid;
+    long long bid;      // bundle within the group
+    bool active;
+
+    __device__ __forceinline__ BundleMap(const SweepParams& p, const GroupDesc& gd, long long bundle)
+        : w(0), valid(0), bid(bundle), active(bundle < gd.n_bundles) {
+        if constexpr (G == 32) {
+            syn[0] = gd.item_base + (active ? bid / p.bps : 0);
+            w = active ? (uint32_t)(bid % p.bps) : 0;
+            sid[0] = p.ids ? p.ids[syn[0]] : p.id0 + (uint32_t)syn[0];
+            const int left = p.C - 32 * (int)w;
+            valid = !active ? 0u : left >= 32 ? 0xFFFFFFFFu : ((1u << left) - 1u);
+        } else {
+#pragma unroll
+            for (int s = 0; s < SLOTS; ++s) {
+                long long li = bid * SLOTS + s;
+                const bool ok = active && li < gd.n;
+                if (!ok) li = bid * SLOTS;  // any in-range syndrome; its bits are masked
+                if (!active) li = 0;
+                syn[s] = gd.item_base + li;
+                sid[s] = p.ids ? p.ids[syn[s]] : p.id0 + (uint32_t)syn[s];
+                if (ok) valid |= ((1u << p.C) - 1u) << (s * G);
+            }
+        }
+    }
+    __device__ __forceinline__ int chain_of(int b) const { return G == 32 ? 32 * (int)w + b : b % G; }
+    __device__ __forceinline__ long long syn_of(int b) const { return G == 32 ? syn[0] : syn[G == 32 ? 0 : b / G]; }
+};
+
+// Bit-sliced start state of a bundle, word by word: the state an earlier
+// launch left, the caller's per-chain frames, or the pure error times the
+// logical that gives chain c the class code c / R (planar code: bit 0 X-bar
+// on row 0, bit 1 Z-bar on column 0; toric code: X1, X2, Z1, Z2).
+template <int G>
+struct StartState {
+    const SweepParams& p;
+    const GroupDesc& gd;
+    const BundleMap<G>& bm;
+    uint32_t lx = 0, lzm = 0, lx2 = 0, lz2 = 0;
+    // per-item arrays of the group: pure errors and frames are laid out per group
+    const uint32_t *e0g, *ifg, *st_in;
+
+    __device__ __forceinline__ StartState(const SweepParams& p_, const GroupDesc& gd_, const BundleMap<G>& bm_)
+        : p(p_), gd(gd_), bm(bm_) {
+        for (int b = 0; b < 32 && !p.init_frames && !p.state_in; ++b) {
+            if (!((bm.valid >> b) & 1u)) continue;
+            const int k = bm.chain_of(b) / p.R;
+            const int l = k ^ p.e0code[bm.syn_of(b)];
+            lx |= (uint32_t)(l & 1) << b;
+            if (p.code) {
+                lx2 |= (uint32_t)((l >> 1) & 1) << b;
+                lzm |= (uint32_t)((l >> 2) & 1) << b;
+                lz2 |= (uint32_t)((l >> 3) & 1) << b;
+            } else {
+                lzm |= (uint32_t)((l >> 1) & 1) << b;
+            }
+        }
+        const int W = gd.W;
+        e0g = p.e0 ? p.e0 + gd.e0_off - (size_t)gd.item_base * 2 * W : nullptr;
+        ifg = p.init_frames ? p.init_frames + gd.frames_off - (size_t)gd.item_base * p.C * 2 * W : nullptr;
+        st_in = p.state_in ? p.state_in + gd.state_off + (size_t)(bm.active ? bm.bid : 0) * 2 * gd.nq : nullptr;
+    }
+
+    // X and Z words of qubit q < nq.
+    __device__ __forceinline__ void word(int q, uint32_t& xw, uint32_t& zw) const {
+        const int W = gd.W, L = gd.L;
+        xw = zw = 0;
+        if (st_in) {
+            if (bm.active) {
+                xw = st_in[q];
+                zw = st_in[gd.nq + q];
+            }
+        } else if (ifg) {
+            for (int b = 0; b < 32; ++b) {
+                if (!((bm.valid >> b) & 1u)) continue;
+                const uint32_t* f = ifg + ((size_t)bm.syn_of(b) * p.C + bm.chain_of(b)) * 2 * W;
+                xw |= ((f[q >> 5] >> (q & 31)) & 1u) << b;
+                zw |= ((f[W + (q >> 5)] >> (q & 31)) & 1u) << b;
+            }
+        } else {
+#pragma unroll
+            for (int s = 0; s < BundleMap<G>::SLOTS; ++s) {
+                const uint32_t vm = G == 32 ? bm.valid : (bm.valid & (((1u << (G & 31)) - 1u) << (s * G)));
+                if (!vm) continue;
+                const uint32_t* e = e0g + (size_t)bm.syn[s] * 2 * W;
+                if ((e[q >> 5] >> (q & 31)) & 1u) xw |= vm;
+                if ((e[W + (q >> 5)] >> (q & 31)) & 1u) zw |= vm;
+            }
+            if (!p.code) {
+                if (q < L) xw ^= lx;                  // row-0 qubits: X-bar
+                if (q % (2 * L - 1) == 0) zw ^= lzm;  // column-0 qubits: Z-bar
+            } else {
+                const int r = q / L;
+                if (r == 1) xw ^= lx;                       // X1: row 1
+                if (q % L == 0 && !(r & 1)) xw ^= lx2;      // X2: column 1, even rows
+                if (q % L == 0 && (r & 1)) zw ^= lzm;       // Z1: column 0, odd rows
+                if (r == 0) zw ^= lz2;                      // Z2: row 0
+            }
+        }
+    }
+};
+
 template <int G, int LAM, bool SCAN, bool IND, bool ACPT, int HM>
 __device__ __forceinline__ void run_unit(const SweepParams& p, const GroupDesc& gd, long long unit,
                                          uint32_t* smem, const ushort4* tab) {
@@ -544,28 +667,9 @@ __device__ __forceinline__ void run_unit(const SweepParams& p, const GroupDesc& 
     uint32_t* binfo = q_items + kQueueCap * kQueueItem;  // per slot: w, sid[SLOTS]
 
     // Syndromes and chains of the bundle.
-    long long syn[SLOTS];
-    uint32_t sid[SLOTS];
-    uint32_t w = 0, valid = 0;
-    // syn[]: the bundle's syndromes as global item indices
-    if constexpr (G == 32) {
-        syn[0] = gd.item_base + (active ? bid / p.bps : 0);
-        w = active ? (uint32_t)(bid % p.bps) : 0;
-        sid[0] = p.ids ? p.ids[syn[0]] : p.id0 + (uint32_t)syn[0];
-        const int left = p.C - 32 * (int)w;
-        valid = !active ? 0u : left >= 32 ? 0xFFFFFFFFu : ((1u << left) - 1u);
-    } else {
-#pragma unroll
-        for (int s = 0; s < SLOTS; ++s) {
-            long long li = bid * SLOTS + s;
-            const bool ok = active && li < gd.n;
-            if (!ok) li = bid * SLOTS;  // any in-range syndrome; its bits are masked
-            if (!active) li = 0;
-            syn[s] = gd.item_base + li;
-            sid[s] = p.ids ? p.ids[syn[s]] : p.id0 + (uint32_t)syn[s];
-            if (ok) valid |= ((1u << p.C) - 1u) << (s * G);
-        }
-    }
+    const BundleMap<G> bm(p, gd, bid);
+    const uint32_t* sid = bm.sid;
+    const uint32_t w = bm.w, valid = bm.valid;
     uint32_t* fx = fixed + (warp * B + slot) * kHeadFixedWords;
     if (sub == 0) {
         binfo[slot * (kMaxSlots + 1)] = w;
@@ -573,70 +677,15 @@ __device__ __forceinline__ void run_unit(const SweepParams& p, const GroupDesc& 
         for (int s = 0; s < SLOTS; ++s) binfo[slot * (kMaxSlots + 1) + 1 + s] = sid[s];
         head_fixed_words<G>(p, sid, w, fx);
     }
-    // chain index and syndrome of bundle bit b
-    auto chain_of = [&](int b) -> int { return G == 32 ? 32 * (int)w + b : b % G; };
-    auto syn_of = [&](int b) -> long long { return G == 32 ? syn[0] : syn[G == 32 ? 0 : b / G]; };
+    auto chain_of = [&](int b) -> int { return bm.chain_of(b); };
+    auto syn_of = [&](int b) -> long long { return bm.syn_of(b); };
 
-    // Start state: pure error times the logical that gives chain c the class
-    // code c / R (bit 0: X-bar on row 0, bit 1: Z-bar on column 0).
-    // (toric code: 4 logical bits X1, X2, Z1, Z2)
-    uint32_t lx = 0, lzm = 0, lx2 = 0, lz2 = 0;
-    for (int b = 0; b < 32 && !p.init_frames && !p.state_in; ++b) {
-        if (!((valid >> b) & 1u)) continue;
-        const int k = chain_of(b) / p.R;
-        const int l = k ^ p.e0code[syn_of(b)];
-        lx |= (uint32_t)(l & 1) << b;
-        if (p.code) {
-            lx2 |= (uint32_t)((l >> 1) & 1) << b;
-            lzm |= (uint32_t)((l >> 2) & 1) << b;
-            lz2 |= (uint32_t)((l >> 3) & 1) << b;
-        } else {
-            lzm |= (uint32_t)((l >> 1) & 1) << b;
-        }
-    }
     const int W = gd.W;
-    // per-item arrays of the group: pure errors and frames are laid out per group
-    const uint32_t* e0g = p.e0 ? p.e0 + gd.e0_off - (size_t)gd.item_base * 2 * W : nullptr;
-    const uint32_t* ifg = p.init_frames ? p.init_frames + gd.frames_off - (size_t)gd.item_base * p.C * 2 * W
-                                        : nullptr;
     uint32_t* cfg = p.chain_frames ? p.chain_frames + gd.frames_off - (size_t)gd.item_base * p.C * 2 * W : nullptr;
-    const uint32_t* st_in = p.state_in ? p.state_in + gd.state_off + (size_t)(active ? bid : 0) * 2 * nq : nullptr;
+    const StartState<G> start(p, gd, bm);
     for (int q = sub; q < nqp; q += LAM) {
-        uint32_t xw = 0, zw = 0;
-        if (q >= nq) {
-            // zero padding
-        } else if (st_in) {
-            if (active) {
-                xw = st_in[q];
-                zw = st_in[nq + q];
-            }
-        } else if (ifg) {
-            for (int b = 0; b < 32; ++b) {
-                if (!((valid >> b) & 1u)) continue;
-                const uint32_t* f = ifg + ((size_t)syn_of(b) * p.C + chain_of(b)) * 2 * W;
-                xw |= ((f[q >> 5] >> (q & 31)) & 1u) << b;
-                zw |= ((f[W + (q >> 5)] >> (q & 31)) & 1u) << b;
-            }
-        } else {
-#pragma unroll
-            for (int s = 0; s < SLOTS; ++s) {
-                const uint32_t vm = G == 32 ? valid : (valid & (((1u << (G & 31)) - 1u) << (s * G)));
-                if (!vm) continue;
-                const uint32_t* e = e0g + (size_t)syn[s] * 2 * W;
-                if ((e[q >> 5] >> (q & 31)) & 1u) xw |= vm;
-                if ((e[W + (q >> 5)] >> (q & 31)) & 1u) zw |= vm;
-            }
-            if (!p.code) {
-                if (q < L) xw ^= lx;                  // row-0 qubits: X-bar
-                if (q % (2 * L - 1) == 0) zw ^= lzm;  // column-0 qubits: Z-bar
-            } else {
-                const int r = q / L;
-                if (r == 1) xw ^= lx;                       // X1: row 1
-                if (q % L == 0 && !(r & 1)) xw ^= lx2;      // X2: column 1, even rows
-                if (q % L == 0 && (r & 1)) zw ^= lzm;       // Z1: column 0, odd rows
-                if (r == 0) zw ^= lz2;                      // Z2: row 0
-            }
-        }
+        uint32_t xw = 0, zw = 0;   // zero padding past nq
+        if (q < nq) start.word(q, xw, zw);
         X[q] = xw;
         Z[q] = zw;
     }
