@@ -348,8 +348,7 @@ struct RaggedGroup {
 struct RaggedLayout {
     std::vector<RaggedGroup> groups;       // in launch order (largest work first)
     std::vector<long long> perm;           // internal index -> caller's index
-    std::vector<long long> src_off, dst_off;
-    std::vector<int32_t> len;
+    std::vector<long long> src_off;        // by the caller's index
     std::vector<uint64_t> samples;         // per internal item
     long long syn_bytes = 0, e0_words = 0, state_words = 0;
     int lam = 0;
@@ -397,16 +396,13 @@ int ragged_layout(surfmcmc_ctx* ctx, const int32_t* Ls, const uint32_t* sweeps, 
     lay.sp.scan = o.scan;
     lay.sp.noise = o.noise;
     energy_table(o, lay.sp.energy);
-    long long dst = 0, item = 0, e0w = 0, stw = 0;
+    long long item = 0, e0w = 0, stw = 0;
     for (auto& g : lay.groups) {
         add_group(lay.sp, g.L, (long long)g.items.size(), item, e0w, 0, stw, lay.lam);
         for (long long i : g.items) {
             lay.perm.push_back(i);
-            lay.dst_off.push_back(dst);
-            lay.len.push_back(n_stabs(g.L));
             lay.samples.push_back(g.sweeps > g.burn ? samples_per_sweep(o, g.L) * o.chains_per_class * (g.sweeps - g.burn)
                                                     : 0);
-            dst += n_stabs(g.L);
         }
         item += (long long)g.items.size();
         e0w += (long long)g.items.size() * 2 * n_words(g.L);
@@ -420,10 +416,8 @@ int ragged_layout(surfmcmc_ctx* ctx, const int32_t* Ls, const uint32_t* sweeps, 
 
 // Device scratch of a ragged run, carved from one base pointer.
 struct RaggedScratch {
-    uint8_t* syn;
     uint32_t* ids;
-    long long *src_off, *dst_off, *perm;
-    int32_t* len;
+    long long *src_off, *perm;
     uint64_t* samples;
     uint32_t* e0;
     int32_t* code;
@@ -434,18 +428,14 @@ struct RaggedScratch {
 
 size_t ragged_scratch(const RaggedLayout& lay, long long n, int Cn, char* base, RaggedScratch* rs) {
     Carver cv;
-    const size_t o_syn = cv.reserve(lay.syn_bytes), o_ids = cv.reserve(n * 4), o_src = cv.reserve(n * 8),
-                 o_dst = cv.reserve(n * 8), o_perm = cv.reserve(n * 8), o_len = cv.reserve(n * 4),
+    const size_t o_ids = cv.reserve(n * 4), o_src = cv.reserve(n * 8), o_perm = cv.reserve(n * 8),
                  o_smp = cv.reserve(n * 8), o_e0 = cv.reserve(lay.e0_words * 4), o_code = cv.reserve(n * 4),
                  o_cs = cv.reserve((size_t)n * Cn * 8), o_st = cv.reserve(lay.state_words * 4),
                  o_ctr = cv.reserve(sizeof(unsigned int));
     if (base && rs) {
-        rs->syn = (uint8_t*)(base + o_syn);
         rs->ids = (uint32_t*)(base + o_ids);
         rs->src_off = (long long*)(base + o_src);
-        rs->dst_off = (long long*)(base + o_dst);
         rs->perm = (long long*)(base + o_perm);
-        rs->len = (int32_t*)(base + o_len);
         rs->samples = (uint64_t*)(base + o_smp);
         rs->e0 = (uint32_t*)(base + o_e0);
         rs->code = (int32_t*)(base + o_code);
@@ -459,39 +449,47 @@ size_t ragged_scratch(const RaggedLayout& lay, long long n, int Cn, char* base, 
 // Copies the host-side tables of the layout to the scratch (synchronously).
 int ragged_upload(surfmcmc_ctx* ctx, const RaggedLayout& lay, long long n, const RaggedScratch& rs, cudaStream_t s) {
     if (n == 0) return SURFMCMC_OK;
-    // src_off is indexed by the caller's index in the gather kernel
     CK(cudaMemcpyAsync(rs.src_off, lay.src_off.data(), n * 8, cudaMemcpyHostToDevice, s));
-    CK(cudaMemcpyAsync(rs.dst_off, lay.dst_off.data(), n * 8, cudaMemcpyHostToDevice, s));
     CK(cudaMemcpyAsync(rs.perm, lay.perm.data(), n * 8, cudaMemcpyHostToDevice, s));
-    CK(cudaMemcpyAsync(rs.len, lay.len.data(), n * 4, cudaMemcpyHostToDevice, s));
     CK(cudaMemcpyAsync(rs.samples, lay.samples.data(), n * 8, cudaMemcpyHostToDevice, s));
     CK(cudaStreamSynchronize(s));
     return SURFMCMC_OK;
 }
 
 // All device work of a ragged run (kernels and memsets only, so that it can
-// be captured into a graph): gather, start frames per group, the sweep
-// segments of every group, decision scattered to the caller's order.
+// be captured into a graph): start frames of every item, the sweep segments
+// of every group, decision scattered to the caller's order.
 int ragged_enqueue(surfmcmc_ctx* ctx, const RaggedLayout& lay, long long n, const surfmcmc_opts& o, double p,
                    uint64_t seed, const uint8_t* syn, const uint32_t* ids, uint32_t id0, const RaggedScratch& rs,
                    int32_t* out_class, uint64_t* out_class_sum, double* out_log_ratio, cudaStream_t s) {
     int rc;
     if (n == 0) return SURFMCMC_OK;
-    CK(launch_gather_rows(n, syn, rs.src_off, rs.dst_off, rs.len, rs.perm, ids, id0, rs.syn, rs.ids, s));
     SweepParams sp = lay.sp;
     sp.ids = rs.ids;
     make_round_keys((uint32_t)seed, (uint32_t)(seed >> 32), &sp.rk);
     std::vector<std::vector<Segment>> plans;
     std::vector<uint32_t> burn;
-    long long syn_off = 0;
+    RaggedStart st;
+    memset(&st, 0, sizeof st);
+    st.n = n;
+    st.n_groups = (int)lay.groups.size();
+    st.src = syn;
+    st.src_off = rs.src_off;
+    st.perm = rs.perm;
+    st.ids = ids;
+    st.id0 = id0;
+    st.e0 = rs.e0;
+    st.code = rs.code;
+    st.ids_out = rs.ids;
     for (size_t g = 0; g < lay.groups.size(); ++g) {
-        const GroupDesc& gd = sp.grp[g];
-        CK(launch_start_frames(rs.syn + syn_off, gd.n, gd.L, rs.e0 + gd.e0_off, rs.code + gd.item_base, s));
-        syn_off += gd.n * n_stabs(gd.L);
+        st.L[g] = sp.grp[g].L;
+        st.item_base[g] = sp.grp[g].item_base;
+        st.e0_off[g] = sp.grp[g].e0_off;
         plans.push_back(plan_segments(lay.groups[g].sweeps, lay.groups[g].burn, o.anneal_stages, o.anneal_beta0,
                                       o.beta_scale, 0));
         burn.push_back(lay.groups[g].burn);
     }
+    CK(launch_start_ragged(st, s));
     SweepIO io;
     io.e0 = rs.e0;
     io.e0code = rs.code;

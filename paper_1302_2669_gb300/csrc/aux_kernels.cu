@@ -1,6 +1,7 @@
 // Syndrome generation, start frames and the per-syndrome decision: the small
-// kernels around the sweep kernel.  One thread per syndrome; frames are kept
-// as packed bit planes in registers/local memory.
+// kernels around the sweep kernel.  One thread per syndrome with the frame as
+// packed bit planes in local memory, but the planar start frames, which stand
+// in front of every decode: one warp per syndrome.
 #include "common.cuh"
 
 namespace surfmcmc {
@@ -80,9 +81,6 @@ __global__ void gen_syndromes_kernel(RoundKeys rk, uint32_t id0, long long n, in
     if (true_class) true_class[i] = class_code(L, ex, ez);
 }
 
-// Pure error: a straight string from every anyon to its nearer absorbing
-// boundary (Sec. III), s-anyons vertically (z string), p-anyons horizontally
-// (x string); ties go up/left.
 // Toric code: syndrome of a frame, its 4-bit class code, and the pure error
 // (defects of each type paired in syndrome order, first with second, ...;
 // a pair joined from the first towards increasing c to the second's
@@ -176,38 +174,106 @@ cudaError_t launch_gen_syndromes_toric(uint64_t seed, uint32_t id0, long long n,
     return cudaGetLastError();
 }
 
-__global__ void start_frames_kernel(const uint8_t* syn, long long n, int L, uint32_t* frames, int32_t* code) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const int W = n_words(L), n2 = 2 * L - 1;
-    uint32_t ex[kMaxWords], ez[kMaxWords];
-    for (int w = 0; w < W; ++w) ex[w] = ez[w] = 0;
-    const uint8_t* s = syn + i * n_stabs(L);
-    int g = 0;
-    for (int a = 0; a < L - 1; ++a)
-        for (int b = 0; b < L; ++b, ++g) {
-            if (!s[g]) continue;
-            const int r = 2 * a + 1, c = 2 * b;
-            if ((r + 1) / 2 <= L - (r + 1) / 2)
-                for (int rr = r - 1; rr >= 0; rr -= 2) flipb(ez, (rr * n2 + c) / 2);
-            else
-                for (int rr = r + 1; rr < n2; rr += 2) flipb(ez, (rr * n2 + c) / 2);
+// Pure error: a straight string from every anyon to its nearer absorbing
+// boundary (Sec. III), s-anyons vertically (z string), p-anyons horizontally
+// (x string); ties go up/left.  One warp per syndrome: the strings touch the
+// qubits of the even grid rows only, lane i holding row 2i of both planes as
+// an L-bit word (bit j: column 2j).  The syndrome's rows become such words by
+// ballots; a z string up (down) from row a covers the rows i <= a (i > a), so
+// the z plane is the suffix (prefix) xor of the row words over the lanes, and
+// the x plane the same over the bits of a word.  (One thread per syndrome
+// walking its strings took 35 us for one syndrome at L = 13 and 300 us at
+// L = 25, all latency.)
+__device__ __forceinline__ void pure_error_rows(int L, const uint8_t* s, int lane, uint32_t& xrow, uint32_t& zrow) {
+    const uint32_t full = 0xffffffffu;
+    uint32_t sx = 0, sz = 0;   // lane a: row a of the sigma_x and of the sigma_z generators
+#pragma unroll 4
+    for (int a = 0; a < L; ++a) {
+        const bool dx = a < L - 1 && lane < L && s[a * L + lane] != 0;
+        const bool dz = lane < L - 1 && s[L * (L - 1) + a * (L - 1) + lane] != 0;
+        const uint32_t wx = __ballot_sync(full, dx), wz = __ballot_sync(full, dz);
+        if (lane == a) {
+            sx = wx;
+            sz = wz;
         }
-    for (int a = 0; a < L; ++a)
-        for (int b = 0; b < L - 1; ++b, ++g) {
-            if (!s[g]) continue;
-            const int r = 2 * a, c = 2 * b + 1;
-            if ((c + 1) / 2 <= L - (c + 1) / 2)
-                for (int cc = c - 1; cc >= 0; cc -= 2) flipb(ex, (r * n2 + cc) / 2);
-            else
-                for (int cc = c + 1; cc < n2; cc += 2) flipb(ex, (r * n2 + cc) / 2);
-        }
-    uint32_t* f = frames + i * 2 * W;
-    for (int w = 0; w < W; ++w) {
-        f[w] = ex[w];
-        f[W + w] = ez[w];
     }
-    if (code) code[i] = class_code(L, ex, ez);
+    // s-anyons of row a go up if 2 (a + 1) <= L
+    uint32_t up = 2 * (lane + 1) <= L ? sx : 0u, down = 2 * (lane + 1) <= L ? 0u : sx;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t u = __shfl_down_sync(full, up, o), d = __shfl_up_sync(full, down, o);
+        if (lane + o < 32) up ^= u;
+        if (lane >= o) down ^= d;
+    }
+    down = __shfl_up_sync(full, down, 1);       // rows below the anyon's
+    zrow = up ^ (lane > 0 ? down : 0u);
+    // p-anyons of column b go left if 2 (b + 1) <= L: bits j <= b; else j > b
+    const uint32_t lmask = (1u << (L / 2)) - 1u;
+    uint32_t left = sz & lmask, right = sz & ~lmask;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        left ^= left >> o;
+        right ^= right << o;
+    }
+    xrow = (left ^ (right << 1)) & ((1u << L) - 1u);
+    zrow = lane < L ? zrow & ((1u << L) - 1u) : 0u;
+    if (lane >= L) xrow = 0u;
+}
+
+// Writes the frame of the row words (f: [2][W]) and returns its class code
+// a + 2b (x parity on column 0, z parity on row 0).  sh: 2 kMaxWords words.
+__device__ __forceinline__ int write_rows(int L, int W, uint32_t xrow, uint32_t zrow, int lane, uint32_t* sh,
+                                          uint32_t* f) {
+    for (int w = lane; w < 2 * W; w += 32) sh[w] = 0u;
+    __syncwarp();
+    if (lane < L) {
+        const int q = lane * (2 * L - 1), w = q >> 5, o = q & 31;
+        const uint64_t x = (uint64_t)xrow << o, z = (uint64_t)zrow << o;
+        atomicOr(&sh[w], (uint32_t)x);
+        atomicOr(&sh[W + w], (uint32_t)z);
+        if (x >> 32) atomicOr(&sh[w + 1], (uint32_t)(x >> 32));
+        if (z >> 32) atomicOr(&sh[W + w + 1], (uint32_t)(z >> 32));
+    }
+    __syncwarp();
+    for (int w = lane; w < 2 * W; w += 32) f[w] = sh[w];
+    const int a = __popc(__ballot_sync(0xffffffffu, xrow & 1u)) & 1;
+    const int b = __popc(__shfl_sync(0xffffffffu, zrow, 0)) & 1;
+    return a + 2 * b;
+}
+
+constexpr int kStartWarps = 4;
+
+__global__ void __launch_bounds__(32 * kStartWarps) start_frames_kernel(const uint8_t* syn, long long n, int L,
+                                                                        uint32_t* frames, int32_t* code) {
+    __shared__ uint32_t sh[kStartWarps][2 * kMaxWords];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, W = n_words(L);
+    const long long i = (long long)blockIdx.x * kStartWarps + warp;
+    if (i >= n) return;
+    uint32_t x, z;
+    pure_error_rows(L, syn + i * n_stabs(L), lane, x, z);
+    const int c = write_rows(L, W, x, z, lane, sh[warp], frames + i * 2 * W);
+    if (code && lane == 0) code[i] = c;
+}
+
+// Ragged batches: pure errors, class codes and ids of every item in one
+// launch, read straight from the caller's rows (item perm[i] of the input at
+// byte src_off[perm[i]]) into group order.
+__global__ void __launch_bounds__(32 * kStartWarps) start_ragged_kernel(const __grid_constant__ RaggedStart p) {
+    __shared__ uint32_t sh[kStartWarps][2 * kMaxWords];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const long long i = (long long)blockIdx.x * kStartWarps + warp;
+    if (i >= p.n) return;
+    int g = 0;
+    while (g + 1 < p.n_groups && i >= p.item_base[g + 1]) ++g;
+    const int L = p.L[g], W = n_words(L);
+    const long long o = p.perm[i];
+    uint32_t x, z;
+    pure_error_rows(L, p.src + p.src_off[o], lane, x, z);
+    const int c = write_rows(L, W, x, z, lane, sh[warp], p.e0 + p.e0_off[g] + (i - p.item_base[g]) * 2 * W);
+    if (lane == 0) {
+        p.code[i] = c;
+        p.ids_out[i] = p.ids ? p.ids[o] : p.id0 + (uint32_t)o;
+    }
 }
 
 // Sec. IV.A decision: S_k = sum over the R chains of class k; the class with
@@ -280,19 +346,6 @@ __global__ void ti_decide_kernel(long long n, int K, int N, double mean0, double
     out_class[i] = best;
     if (out_log_z)
         for (int k = 0; k < K; ++k) out_log_z[i * K + k] = -__dsub_rn(I[k], I[best]);
-}
-
-// Ragged batches: copies the caller's syndrome rows (item perm[i] of the
-// input) into group order and sets the internal ids.
-__global__ void gather_rows_kernel(long long n, const uint8_t* src, const long long* src_off, const long long* dst_off,
-                                   const int32_t* len, const long long* perm, const uint32_t* ids, uint32_t id0,
-                                   uint8_t* dst, uint32_t* ids_out) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const uint8_t* a = src + src_off[perm[i]];
-    uint8_t* b = dst + dst_off[i];
-    for (int k = 0; k < len[i]; ++k) b[k] = a[k];
-    ids_out[i] = ids ? ids[perm[i]] : id0 + (uint32_t)perm[i];
 }
 
 // Early stop, after a chunk of sweeps: item i of the active set (caller's
@@ -499,12 +552,9 @@ cudaError_t launch_compact(long long n, const int32_t* keep, long long* pos, lon
     return cudaGetLastError();
 }
 
-cudaError_t launch_gather_rows(long long n, const uint8_t* src, const long long* src_off, const long long* dst_off,
-                               const int32_t* len, const long long* perm, const uint32_t* ids, uint32_t id0,
-                               uint8_t* dst, uint32_t* ids_out, cudaStream_t s) {
-    if (n == 0) return cudaSuccess;
-    gather_rows_kernel<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(n, src, src_off, dst_off, len, perm, ids, id0, dst,
-                                                                   ids_out);
+cudaError_t launch_start_ragged(const RaggedStart& p, cudaStream_t s) {
+    if (p.n == 0) return cudaSuccess;
+    start_ragged_kernel<<<(unsigned)((p.n + kStartWarps - 1) / kStartWarps), 32 * kStartWarps, 0, s>>>(p);
     return cudaGetLastError();
 }
 
@@ -542,7 +592,8 @@ cudaError_t launch_start_frames(const uint8_t* syn, long long n, int L, uint32_t
     if (toric)
         start_frames_toric_kernel<<<(unsigned)((n + bs - 1) / bs), bs, 0, s>>>(syn, n, L, frames, code);
     else
-        start_frames_kernel<<<(unsigned)((n + bs - 1) / bs), bs, 0, s>>>(syn, n, L, frames, code);
+        start_frames_kernel<<<(unsigned)((n + kStartWarps - 1) / kStartWarps), 32 * kStartWarps, 0, s>>>(syn, n, L,
+                                                                                                         frames, code);
     return cudaGetLastError();
 }
 

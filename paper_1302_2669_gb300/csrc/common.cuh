@@ -248,6 +248,23 @@ struct SweepParams {
     GroupDesc grp[kMaxGroups];
 };
 
+// Start of a ragged run: where every item's row is and where its pure error
+// goes (groups as in SweepParams).
+struct RaggedStart {
+    long long n;
+    int n_groups;
+    int L[kMaxGroups];
+    long long item_base[kMaxGroups], e0_off[kMaxGroups];
+    const uint8_t* src;
+    const long long* src_off;   // by the caller's index
+    const long long* perm;      // caller's index of internal item i
+    const uint32_t* ids;        // by the caller's index, or NULL (id0 + index)
+    uint32_t id0;
+    uint32_t* e0;
+    int32_t* code;              // by internal item
+    uint32_t* ids_out;
+};
+
 struct DecideParams {
     long long n;
     int K, R;
@@ -282,9 +299,7 @@ cudaError_t launch_start_frames(const uint8_t* syn, long long n, int L, uint32_t
 cudaError_t launch_gen_syndromes_toric(uint64_t seed, uint32_t id0, long long n, int L, double p, uint8_t* syn,
                                        int32_t* true_class, cudaStream_t s);
 cudaError_t launch_decide(const DecideParams& p, cudaStream_t s);
-cudaError_t launch_gather_rows(long long n, const uint8_t* src, const long long* src_off, const long long* dst_off,
-                               const int32_t* len, const long long* perm, const uint32_t* ids, uint32_t id0,
-                               uint8_t* dst, uint32_t* ids_out, cudaStream_t s);
+cudaError_t launch_start_ragged(const RaggedStart& p, cudaStream_t s);
 cudaError_t launch_class_means(long long n, int K, int R, int N, int j, uint64_t samples, const uint64_t* chain_sum,
                                double* mean, cudaStream_t s);
 cudaError_t launch_ti_decide(long long n, int K, int N, double mean0, double h3, double* mean, int32_t* out_class,

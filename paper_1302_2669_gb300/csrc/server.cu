@@ -135,7 +135,16 @@ void worker_main(surfmcmc_server* s) {
                     free_slot = &sl;
                     break;
                 }
-            if (free_slot && !s->pending.empty()) {
+            // Memory first: with requests waiting and a slot free, not even the
+            // next request's scratch may fit next to the batches in flight;
+            // that wait is counted once, whether or not the batch would be
+            // complete yet.
+            const size_t budget = (size_t)s->sopts.memory_budget;
+            const bool blocked = free_slot && !s->pending.empty() && budget > 0 && s->in_flight_bytes > 0 &&
+                                 s->in_flight_bytes + kBatchBaseBytes + request_bytes(s->pending.front().L, R) > budget;
+            if (blocked && !s->waiting_for_memory) ++s->memory_stalls;
+            s->waiting_for_memory = blocked;
+            if (free_slot && !s->pending.empty() && !blocked) {
                 // a partial batch waits up to max_wait_us for company
                 const double waited = std::chrono::duration<double, std::micro>(
                                           Clock::now() - s->pending.front().t_submit).count();
@@ -144,7 +153,6 @@ void worker_main(surfmcmc_server* s) {
                     // the batch: the longest prefix of the queue of at most
                     // max_batch requests whose scratch fits the memory budget
                     // next to the batches in flight (at least one request)
-                    const size_t budget = (size_t)s->sopts.memory_budget;
                     size_t need = kBatchBaseBytes;
                     int64_t k = 0;
                     for (auto it = s->pending.begin(); it != s->pending.end() && k < s->sopts.max_batch; ++it) {
@@ -153,23 +161,15 @@ void worker_main(surfmcmc_server* s) {
                         need += b;
                         ++k;
                     }
-                    if (budget > 0 && s->in_flight_bytes > 0 && s->in_flight_bytes + need > budget) {
-                        // not even one request fits: wait for a batch in flight
-                        // to finish (counted once per wait)
-                        if (!s->waiting_for_memory) ++s->memory_stalls;
-                        s->waiting_for_memory = true;
-                    } else {
-                        s->waiting_for_memory = false;
-                        batch.reserve((size_t)k);
-                        for (int64_t i = 0; i < k; ++i) {
-                            batch.push_back(std::move(s->pending.front()));
-                            s->pending.pop_front();
-                        }
-                        free_slot->scratch = need;
-                        s->in_flight_bytes += need;
-                        s->admitted += k;
-                        ++s->batches;
+                    batch.reserve((size_t)k);
+                    for (int64_t i = 0; i < k; ++i) {
+                        batch.push_back(std::move(s->pending.front()));
+                        s->pending.pop_front();
                     }
+                    free_slot->scratch = need;
+                    s->in_flight_bytes += need;
+                    s->admitted += k;
+                    ++s->batches;
                 }
             }
             if (batch.empty()) {
