@@ -284,6 +284,8 @@ cudaError_t launch_sweep_flips(const SweepParams& p, int lanes_per_bundle, cudaS
 // The launch on a kernel with its digit-plane modes compiled in;
 // cudaErrorNotSupported (nothing launched) where there is none.
 cudaError_t launch_sweep_modes(const SweepParams& p, int lanes_per_bundle, cudaStream_t s);
+// Random scan (sweep_scan.cu).
+cudaError_t launch_sweep_scan(const SweepParams& p, cudaStream_t s);
 // The launch with one block per bundle (colour sweeps without accept counts).
 cudaError_t launch_sweep_wide(const SweepParams& p, cudaStream_t s);
 cudaError_t prepare_sweep_flips(const SweepParams& p, int lanes_per_bundle);

@@ -16,16 +16,16 @@ long long sweep_units(long long n_bundles, int lam) { return (n_bundles + (long 
 
 // Sets the kernel's shared-memory limit ahead of a stream capture.
 cudaError_t prepare_sweep(const SweepParams& p, int lam) {
+    if (p.scan || p.wide) return cudaSuccess;   // their launchers raise it themselves
     return p.noise == 1 ? prepare_sweep_flips(p, lam) : prepare_noise<false>(p, lam);
 }
 
 cudaError_t launch_sweep(const SweepParams& p, int lam, cudaStream_t s) {
+    if (p.scan) return launch_sweep_scan(p, s);
     if (p.wide) return launch_sweep_wide(p, s);
     // kernels with the launch's digit-plane modes compiled in, where they exist
     const cudaError_t e = launch_sweep_modes(p, lam, s);
     if (e != cudaErrorNotSupported) return e;
-    // the general channel (noise 2) runs only in random scan, which reads the
-    // energy table and not the template's noise model
     return p.noise == 1 ? launch_sweep_flips(p, lam, s) : launch_noise<false>(p, lam, s);
 }
 

@@ -1,6 +1,6 @@
 // The Metropolis sweep kernel (Sec. IV / IV.A, parallelised as in Sec. V),
-// templated on the chain layout, the lanes per bundle, the scan mode and the
-// noise model; sweep.cu and sweep_flips.cu instantiate it for depolarizing
+// templated on the chain layout, the lanes per bundle and the noise model;
+// sweep.cu and sweep_flips.cu instantiate it for depolarizing
 // noise and for independent bit and phase flips.
 //
 // Data layout.  Chains are bit-sliced: a "bundle" holds 32 chains, and each
@@ -449,37 +449,9 @@ __host__ __device__ __forceinline__ int warp_aux_words(int bundles) {
     return 1 + kQueueCap * kQueueItem + bundles * (kMaxSlots + 1);
 }
 
-// Support of generator g in the syndrome order (sigma_x block row-major over
-// (i, j) at grid point (2i+1, 2j), then the sigma_z block at (2i, 2j+1)):
-// up, down, left, right neighbours, a missing one replaced by the dummy slot
-// (nq for sigma_x generators, nq + 1 for sigma_z).  Returns 0 for sigma_x
-// (flips the X plane), 1 for sigma_z.
-__device__ __forceinline__ int generator_support(int L, int g, int q[4]) {
-    const int nx = L * (L - 1), n = 2 * L - 1, nq = n_qubits(L);
-    int r, c, type;
-    if (g < nx) {
-        const int i = g / L;
-        r = 2 * i + 1;
-        c = 2 * (g - i * L);
-        type = 0;
-    } else {
-        const int h = g - nx, i = h / (L - 1);
-        r = 2 * i;
-        c = 2 * (h - i * (L - 1)) + 1;
-        type = 1;
-    }
-    const int dummy = nq + type, base = r * n + c;
-    q[0] = r > 0 ? (base - n) / 2 : dummy;
-    q[1] = r < n - 1 ? (base + n) / 2 : dummy;
-    q[2] = c > 0 ? (base - 1) / 2 : dummy;
-    q[3] = c < n - 1 ? (base + 1) / 2 : dummy;
-    return type;
-}
-
 // One unit: the bundles of group g handled by this block (warps x 32/LAM
 // bundles); every warp runs its bundles' chains from gd.t_begin to gd.t_end.
-// SCAN (with LAM = 32, one chain per lane): random-scan steps instead of
-// colour sweeps, on the same bit-sliced frames.  IND: independent bit and
+// IND: independent bit and
 // phase flips (n = |x| + |z|, every real qubit movable) instead of
 // depolarizing noise (n = |x or z|, a qubit movable when its other part is 0).
 // Per-lane count of the accepted proposals of its bundle's chains (bit b =
@@ -644,7 +616,7 @@ struct StartState {
     }
 };
 
-template <int G, int LAM, bool SCAN, bool IND, bool ACPT, int HM>
+template <int G, int LAM, bool IND, bool ACPT, int HM>
 __device__ __forceinline__ void run_unit(const SweepParams& p, const GroupDesc& gd, long long unit,
                                          uint32_t* smem, const ushort4* tab) {
     constexpr int B = 32 / LAM;                       // bundles per warp
@@ -710,58 +682,6 @@ __device__ __forceinline__ void run_unit(const SweepParams& p, const GroupDesc& 
     uint32_t since_flush = 0;
     __syncwarp();
 
-    int scan_n = 0;  // random scan: the lane's chain's n at the end
-    if constexpr (SCAN) {
-        static_assert(LAM == 32, "random scan runs one chain per lane");
-        // Sec. IV as written: each step draws one generator g = floor(w0
-        // n_stab / 2^32) and applies it when Delta n <= 0 or w1 < T[Delta n]
-        // (Philox counter (id, chain, t, step)); n is summed after every
-        // step.  Lane b owns bit b of the bundle's words and flips only it.
-        const int b = lane;
-        const bool mine = (valid >> b) & 1u;
-        const uint32_t bit = 1u << b;
-        const uint32_t my_sid = sid[G == 32 ? 0 : b / G];
-        const uint32_t chain = (uint32_t)chain_of(b);
-        const int ns = geo_nstab(p.code, L);
-        // energy of a qubit's Pauli, index x + 2z (I, X, Z, Y): the noise
-        // model's table (depolarizing 0 1 1 1, flips 0 1 1 2, general)
-        const int E0 = p.energy[0], E1 = p.energy[1], E2 = p.energy[2], E3 = p.energy[3];
-        auto energy = [&](uint32_t x, uint32_t z) { return x ? (z ? E3 : E1) : (z ? E2 : E0); };
-        int n = 0;
-        for (int q = 0; q < nq; ++q) n += energy((X[q] >> b) & 1u, (Z[q] >> b) & 1u);
-        uint64_t sum = 0, n_acc = 0;
-        const int n_x = p.code ? L * L : L * (L - 1);   // sigma_x generators come first
-        for (uint32_t t = gd.t_begin; t < gd.t_end; ++t) {
-            const bool sample = t >= gd.burn_in;
-            for (int step = 0; step < ns; ++step) {
-                const uint4 r = philox10(make_uint4(my_sid, chain, t, (uint32_t)step), p.rk);
-                const int g = (int)__umulhi(r.x, (uint32_t)ns);
-                const ushort4 sp = tab[g];
-                const int q[4] = {sp.x, sp.y, sp.z, sp.w};
-                const int type = g >= n_x;
-                uint32_t* own = type == 0 ? X : Z;
-                const uint32_t* oth = type == 0 ? Z : X;
-                int dn = 0;
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    if (q[k] >= nq) continue;  // dummy slot of a weight-3 generator
-                    const uint32_t o = (own[q[k]] >> b) & 1u, t2 = (oth[q[k]] >> b) & 1u;
-                    dn += type == 0 ? energy(o ^ 1u, t2) - energy(o, t2) : energy(t2, o ^ 1u) - energy(t2, o);
-                }
-                if (mine && (dn <= 0 || (uint64_t)r.y < p.T[dn])) {
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) atomicXor(&own[q[k]], bit);
-                    n += dn;
-                    ++n_acc;
-                }
-                if (sample) sum += (uint64_t)n;
-            }
-        }
-        if (mine && p.chain_sum) p.chain_sum[ci_of(b)] += sum;
-        if (mine && p.accepts) p.accepts[ci_of(b)] += n_acc;   // one lane per chain
-        scan_n = n;
-        __syncwarp();
-    } else
     for (uint32_t t = gd.t_begin; t < gd.t_end; ++t) {
 #pragma unroll 1
         for (int col = 0; col < 4; ++col) {
@@ -893,13 +813,13 @@ __device__ __forceinline__ void run_unit(const SweepParams& p, const GroupDesc& 
         }
     }
     uint32_t cnt[kCountBits] = {};
-    if constexpr (!SCAN) recount<LAM, IND>(X, Z, nqp, sub, cnt);
+    recount<LAM, IND>(X, Z, nqp, sub, cnt);
 #pragma unroll
     for (int j = 0; j < NJ; ++j) {
         const int b = sub + j * LAM;
         if (!((valid >> b) & 1u)) continue;
         const size_t ci = (size_t)syn_of(b) * p.C + chain_of(b);
-        if (p.chain_n) p.chain_n[ci] = SCAN ? scan_n : (int32_t)bit_of(cnt, b);
+        if (p.chain_n) p.chain_n[ci] = (int32_t)bit_of(cnt, b);
         if (cfg) {
             uint32_t* f = cfg + ci * 2 * W;
             for (int wi = 0; wi < W; ++wi) {
@@ -922,7 +842,7 @@ __device__ __forceinline__ void run_unit(const SweepParams& p, const GroupDesc& 
 // fill its warps) first by its index, then from a queue counter, in the order
 // the host arranged (largest work first), and rebuilds the support table in
 // shared memory when the group's code size changes.
-template <int G, int LAM, bool SCAN, bool IND, bool ACPT, int HM = 0>
+template <int G, int LAM, bool IND, bool ACPT, int HM = 0>
 __global__ void __launch_bounds__(128, sweep_blocks_per_sm(G)) sweep_kernel(const __grid_constant__ SweepParams p) {
     extern __shared__ __align__(16) uint32_t smem[];
     __shared__ long long s_unit;
@@ -939,18 +859,12 @@ __global__ void __launch_bounds__(128, sweep_blocks_per_sm(G)) sweep_kernel(cons
         while (g + 1 < p.n_groups && u >= p.grp[g + 1].unit_base) ++g;
         const GroupDesc& gd = p.grp[g];
         if (g != cur) {
-            // support table: colour-major for sweeps, syndrome order for
-            // random scan (4 nc = n_stab entries either way)
+            // support table, colour-major (4 nc = n_stab entries)
             for (int idx = threadIdx.x; idx < 4 * gd.nc; idx += blockDim.x) {
                 int q[4];
-                if constexpr (SCAN) {
-                    if (p.code) toric_generator_support(gd.L, idx, q);
-                    else generator_support(gd.L, idx, q);
-                } else {
-                    const int col = idx / gd.nc, m = idx - col * gd.nc;
-                    if (p.code) toric_colour_support(gd.L, col, m, q);
-                    else colour_support(gd.L, col, m, q);
-                }
+                const int col = idx / gd.nc, m = idx - col * gd.nc;
+                if (p.code) toric_colour_support(gd.L, col, m, q);
+                else colour_support(gd.L, col, m, q);
                 // dummy slots (nq, nq + 1) sit after the zero-padded planes
                 const int nq = gd.nq, shift = padded_nq(nq, LAM) - nq;
 #pragma unroll
@@ -962,7 +876,7 @@ __global__ void __launch_bounds__(128, sweep_blocks_per_sm(G)) sweep_kernel(cons
             cur = g;
             __syncthreads();
         }
-        run_unit<G, LAM, SCAN, IND, ACPT, HM>(p, gd, u - gd.unit_base, smem, tab);
+        run_unit<G, LAM, IND, ACPT, HM>(p, gd, u - gd.unit_base, smem, tab);
         __syncthreads();
         if (!p.unit_counter) break;
     }
@@ -990,14 +904,14 @@ struct SmemLimit {
     }
 };
 
-template <int G, int LAM, bool SCAN, bool IND, bool ACPT = false, int HM = 0>
+template <int G, int LAM, bool IND, bool ACPT = false, int HM = 0>
 static cudaError_t launch_t(const SweepParams& p, cudaStream_t s) {
     const size_t smem = sweep_smem_bytes(p.grp_nq_max, p.grp_nc_max, LAM) +
                         (ACPT ? (size_t)kWarps * kAcptWordsPerWarp * 4 : 0);
     static SmemLimit limit;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = limit.ensure(sweep_kernel<G, LAM, SCAN, IND, ACPT, HM>, dev, smem);
+    if (e == cudaSuccess) e = limit.ensure(sweep_kernel<G, LAM, IND, ACPT, HM>, dev, smem);
     if (e != cudaSuccess) return e;
     if (p.total_units == 0) return cudaSuccess;
     long long blocks = p.total_units;
@@ -1006,7 +920,7 @@ static cudaError_t launch_t(const SweepParams& p, cudaStream_t s) {
         int sms = 0, per_sm = 0;
         e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (e == cudaSuccess)
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sweep_kernel<G, LAM, SCAN, IND, ACPT, HM>, 32 * kWarps,
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sweep_kernel<G, LAM, IND, ACPT, HM>, 32 * kWarps,
                                                               smem);
         if (e != cudaSuccess) return e;
         int bps = per_sm > 0 ? per_sm : 1;
@@ -1016,26 +930,25 @@ static cudaError_t launch_t(const SweepParams& p, cudaStream_t s) {
         e = cudaMemsetAsync(p.unit_counter, 0, sizeof(unsigned int), s);
         if (e != cudaSuccess) return e;
     }
-    sweep_kernel<G, LAM, SCAN, IND, ACPT, HM><<<(unsigned)blocks, 32 * kWarps, smem, s>>>(p);
+    sweep_kernel<G, LAM, IND, ACPT, HM><<<(unsigned)blocks, 32 * kWarps, smem, s>>>(p);
     return cudaGetLastError();
 }
 
-template <int G, int LAM, bool SCAN, bool IND>
+template <int G, int LAM, bool IND>
 static cudaError_t prepare_t(const SweepParams& p) {
     const size_t smem = sweep_smem_bytes(p.grp_nq_max, p.grp_nc_max, LAM);
-    return cudaFuncSetAttribute(sweep_kernel<G, LAM, SCAN, IND, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    return cudaFuncSetAttribute(sweep_kernel<G, LAM, IND, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)smem);
 }
 
 template <int G, bool IND>
 static cudaError_t prepare_g(const SweepParams& p, int lam) {
-    if (p.scan) return lam == 32 ? prepare_t<G, 32, true, IND>(p) : cudaErrorInvalidValue;
     switch (lam) {
-        case 2: return prepare_t<G, 2, false, IND>(p);
-        case 4: return prepare_t<G, 4, false, IND>(p);
-        case 8: return prepare_t<G, 8, false, IND>(p);
-        case 16: return prepare_t<G, 16, false, IND>(p);
-        case 32: return prepare_t<G, 32, false, IND>(p);
+        case 2: return prepare_t<G, 2, IND>(p);
+        case 4: return prepare_t<G, 4, IND>(p);
+        case 8: return prepare_t<G, 8, IND>(p);
+        case 16: return prepare_t<G, 16, IND>(p);
+        case 32: return prepare_t<G, 32, IND>(p);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -1053,15 +966,14 @@ static cudaError_t prepare_noise(const SweepParams& p, int lam) {
 
 template <int G, bool IND>
 static cudaError_t launch_g(const SweepParams& p, int lam, cudaStream_t s) {
-    if (p.scan) return lam == 32 ? launch_t<G, 32, true, IND>(p, s) : cudaErrorInvalidValue;
     // colour sweeps that count accepted proposals: one lane split only
-    if (p.accepts) return lam == 32 ? launch_t<G, 32, false, IND, true>(p, s) : cudaErrorInvalidValue;
+    if (p.accepts) return lam == 32 ? launch_t<G, 32, IND, true>(p, s) : cudaErrorInvalidValue;
     switch (lam) {
-        case 2: return launch_t<G, 2, false, IND>(p, s);
-        case 4: return launch_t<G, 4, false, IND>(p, s);
-        case 8: return launch_t<G, 8, false, IND>(p, s);
-        case 16: return launch_t<G, 16, false, IND>(p, s);
-        case 32: return launch_t<G, 32, false, IND>(p, s);
+        case 2: return launch_t<G, 2, IND>(p, s);
+        case 4: return launch_t<G, 4, IND>(p, s);
+        case 8: return launch_t<G, 8, IND>(p, s);
+        case 16: return launch_t<G, 16, IND>(p, s);
+        case 32: return launch_t<G, 32, IND>(p, s);
         default: return cudaErrorInvalidValue;
     }
 }

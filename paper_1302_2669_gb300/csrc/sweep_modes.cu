@@ -12,9 +12,9 @@ namespace surfmcmc {
 template <int G, int HM>
 static cudaError_t launch_hm(const SweepParams& p, int lam, cudaStream_t s) {
     switch (lam) {
-        case 8: return launch_t<G, 8, false, false, false, HM>(p, s);
-        case 16: return launch_t<G, 16, false, false, false, HM>(p, s);
-        case 32: return launch_t<G, 32, false, false, false, HM>(p, s);
+        case 8: return launch_t<G, 8, false, false, HM>(p, s);
+        case 16: return launch_t<G, 16, false, false, HM>(p, s);
+        case 32: return launch_t<G, 32, false, false, HM>(p, s);
         default: return cudaErrorNotSupported;
     }
 }
