@@ -33,6 +33,11 @@ struct surfmcmc_ctx {
     std::map<std::pair<int, int>, Tuned> tuned;  // (L, chains per class) -> launch shape
     std::vector<std::pair<cudaEvent_t, cudaEvent_t>> pending;  // recorded around sweep launches
     std::vector<std::pair<cudaEvent_t, cudaEvent_t>> spare;
+    // side streams of decode_ti's grid points and their events (start, done);
+    // created on first use
+    std::vector<cudaStream_t> side;
+    std::vector<cudaEvent_t> side_done;
+    cudaEvent_t side_start = nullptr;
 };
 
 namespace {
@@ -99,6 +104,26 @@ int ensure_arena(surfmcmc_ctx* ctx, size_t bytes) {
     size_t want = bytes + bytes / 4;
     CK(cudaMalloc(&ctx->arena, want));
     ctx->arena_bytes = want;
+    return SURFMCMC_OK;
+}
+
+// Side streams of decode_ti, at most kTiStreams, with an event each.
+constexpr int kTiStreams = 16;
+
+int ensure_side(surfmcmc_ctx* ctx, int count) {
+    if (!ctx->side_start) CK(cudaEventCreateWithFlags(&ctx->side_start, cudaEventDisableTiming));
+    while ((int)ctx->side.size() < count) {
+        cudaStream_t st;
+        cudaEvent_t ev;
+        CK(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+        const cudaError_t e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
+        if (e != cudaSuccess) {
+            cudaEventDestroy(ev);
+            CK(e);
+        }
+        ctx->side.push_back(st);
+        ctx->side_done.push_back(ev);
+    }
     return SURFMCMC_OK;
 }
 
@@ -617,6 +642,12 @@ void surfmcmc_destroy(surfmcmc_ctx* ctx) {
         cudaDeviceSynchronize();
         cudaFree(ctx->arena);
     }
+    for (cudaStream_t st : ctx->side) {
+        cudaStreamSynchronize(st);
+        cudaStreamDestroy(st);
+    }
+    for (cudaEvent_t e : ctx->side_done) cudaEventDestroy(e);
+    if (ctx->side_start) cudaEventDestroy(ctx->side_start);
     for (auto* v : {&ctx->pending, &ctx->spare})
         for (auto& e : *v) {
             cudaEventDestroy(e.first);
@@ -913,11 +944,17 @@ int surfmcmc_decode_ti(surfmcmc_ctx* ctx, const uint8_t* syndromes, int64_t n, i
     sp.scan = o.scan;
     sp.noise = o.noise;
     energy_table(o, sp.energy);
-    // a batch too small to fill the device gets more lanes per bundle (the
-    // results do not depend on the lane split)
-    lam = widen_lanes(ctx, L, o.lanes_per_bundle, lam, bundles_of(sp, n), sp.G, toric);
+    // The grid points are independent: S of them run at a time on streams of
+    // their own, enough to fill the device twice over, and the launch shape
+    // follows the bundles of all of them.  (One after the other, the 4,096
+    // syndromes of an L = 9 batch filled a third of the device and its lanes
+    // were widened to 56 % of use: 90.7 ms against 37.0.)
+    const long long nb = bundles_of(sp, n);
+    lam = widen_lanes(ctx, L, o.lanes_per_bundle, lam, nb * (N - 1), sp.G, toric);
     add_group(sp, L, n, 0, 0, 0, 0, lam);
-    sp.wide = take_wide(ctx, o, sp);
+    sp.wide = o.lanes_per_bundle ? 0 : wide_batch(ctx->sms, sp, N - 1);
+    const long long fill = 2LL * ctx->sms * sweep_blocks_per_sm(sp.G), units = std::max(1LL, sweep_units(nb, lam));
+    const int S = (int)std::max(1LL, std::min({(long long)(N - 1), (long long)kTiStreams, (fill + units - 1) / units}));
     const std::vector<Segment> segs0 = plan_segments(o, o.beta_scale, 0);
     const int W = geo_words(toric, L), nq = geo_nq(toric, L);
 
@@ -928,37 +965,60 @@ int surfmcmc_decode_ti(surfmcmc_ctx* ctx, const uint8_t* syndromes, int64_t n, i
     plan(b_lz, out_log_z, out_log_z ? (size_t)n * K * 8 : 0, cv);
     const bool mean_scratch = !out_mean || !is_device_ptr(out_mean);
     const size_t off_mean = mean_scratch ? cv.reserve((size_t)n * K * N * 8) : 0;
-    const size_t off_chs = cv.reserve((size_t)n * Cn * 8);
+    // per stream: chain sums, bundle state, work queue
+    std::vector<size_t> off_chs(S), off_state(S), off_ctr(S);
+    for (int i = 0; i < S; ++i) {
+        off_chs[i] = cv.reserve((size_t)n * Cn * 8);
+        off_state[i] = segs0.size() > 1 ? cv.reserve((size_t)sp.grp[0].n_bundles * 2 * nq * 4) : 0;
+        off_ctr[i] = cv.reserve(sizeof(unsigned int));
+    }
     const size_t off_e0 = cv.reserve((size_t)n * 2 * W * 4);
     const size_t off_code = cv.reserve((size_t)n * 4);
-    const size_t off_state = segs0.size() > 1 ? cv.reserve((size_t)sp.grp[0].n_bundles * 2 * nq * 4) : 0;
-    const size_t off_ctr = cv.reserve(sizeof(unsigned int));
     if ((rc = ensure_arena(ctx, cv.off))) return rc;
+    if (S > 1 && (rc = ensure_side(ctx, S))) return rc;
     for (Buf* b : {&b_syn, &b_cls, &b_lz}) bind(*b, ctx);
     char* base = (char*)ctx->arena;
     double* mean = mean_scratch ? (double*)(base + off_mean) : out_mean;
-    uint64_t* chain_sum = (uint64_t*)(base + off_chs);
     uint32_t* e0 = (uint32_t*)(base + off_e0);
     int32_t* code = (int32_t*)(base + off_code);
-    uint32_t* state = segs0.size() > 1 ? (uint32_t*)(base + off_state) : nullptr;
-    unsigned int* ctr = (unsigned int*)(base + off_ctr);
 
     if ((rc = copy_in(ctx, b_syn, s))) return rc;
     CK(launch_start_frames((const uint8_t*)b_syn.dev, n, L, e0, code, s, toric));
     const uint64_t samples = samples_per_sweep(o, L) * R * (o.n_sweeps - o.burn_in);
-    for (int j = 1; j < N; ++j) {
-        // grid point j: beta_j = beta* j/(N-1), randomness keyed by seed + j
+    auto grid_point = [&](int j, int i, cudaStream_t st) -> int {
+        // beta_j = beta* j/(N-1), randomness keyed by seed + j
         const double bs = o.beta_scale * (double)j / (double)(N - 1);
         const uint64_t sj = seed + (uint64_t)j;
         make_round_keys((uint32_t)sj, (uint32_t)(sj >> 32), &sp.rk);
         SweepIO io;
         io.e0 = e0;
         io.e0code = code;
-        io.chain_sum = chain_sum;
-        io.state = state;
-        io.unit_counter = ctr;
-        if ((rc = run_segments(ctx, sp, plan_segments(o, bs, 0), o.burn_in, p, lam, io, s))) return rc;
-        CK(launch_class_means(n, K, R, N, j, samples, chain_sum, mean, s));
+        io.chain_sum = (uint64_t*)(base + off_chs[i]);
+        io.state = segs0.size() > 1 ? (uint32_t*)(base + off_state[i]) : nullptr;
+        io.unit_counter = (unsigned int*)(base + off_ctr[i]);
+        const int r = run_segments(ctx, sp, plan_segments(o, bs, 0), o.burn_in, p, lam, io, st);
+        if (r) return r;
+        CK(launch_class_means(n, K, R, N, j, samples, io.chain_sum, mean, st));
+        return SURFMCMC_OK;
+    };
+    if (S == 1) {
+        for (int j = 1; j < N; ++j)
+            if ((rc = grid_point(j, 0, s))) return rc;
+    } else {
+        // fork from the caller's stream and join it again, also after an error
+        // (the side streams work on the context's scratch)
+        CK(cudaEventRecord(ctx->side_start, s));
+        rc = SURFMCMC_OK;
+        int forked = 0;
+        for (; forked < S && !rc; ++forked)
+            if (cudaStreamWaitEvent(ctx->side[forked], ctx->side_start, 0) != cudaSuccess)
+                rc = fail(ctx, SURFMCMC_ECUDA, "side stream: %s", cudaGetErrorString(cudaGetLastError()));
+        for (int j = 1; j < N && !rc; ++j) rc = grid_point(j, (j - 1) % S, ctx->side[(j - 1) % S]);
+        for (int i = 0; i < forked; ++i)
+            if ((cudaEventRecord(ctx->side_done[i], ctx->side[i]) != cudaSuccess ||
+                 cudaStreamWaitEvent(s, ctx->side_done[i], 0) != cudaSuccess) && !rc)
+                rc = fail(ctx, SURFMCMC_ECUDA, "side stream: %s", cudaGetErrorString(cudaGetLastError()));
+        if (rc) return rc;
     }
     uint64_t T[33];
     double beta_bar;

@@ -140,11 +140,12 @@ inline int widen_lanes_for(int sms, int L, int lam, long long n_bundles, int G, 
 // multiprocessor it is the faster one at every size measured (L = 5: 211
 // against 333 us for 60 sweeps, L = 25: 1618 against 1766); from 8 on it is
 // not.  The budget shares a multiprocessor's 1024 threads (64 registers
-// each) among its bundles.
-inline int wide_batch(int sms, const SweepParams& sp) {
+// each) among its bundles.  at_once: launches of this shape that run at the
+// same time.
+inline int wide_batch(int sms, const SweepParams& sp, int at_once = 1) {
     if (sp.scan || sp.accepts || sms <= 0) return 0;
     long long bundles = 0;
-    for (int g = 0; g < sp.n_groups; ++g) bundles += sp.grp[g].n_bundles;
+    for (int g = 0; g < sp.n_groups; ++g) bundles += sp.grp[g].n_bundles * at_once;
     if (bundles > 4LL * sms) return 0;
     const long long per_sm = (bundles + sms - 1) / sms;
     return (int)(1024 / (per_sm < 1 ? 1 : per_sm > 4 ? 4 : per_sm));
