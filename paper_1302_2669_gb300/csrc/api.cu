@@ -167,25 +167,25 @@ int check_common(surfmcmc_ctx* ctx, int64_t n, int32_t L, uint32_t id0) {
     return SURFMCMC_OK;
 }
 
-// Lanes per bundle of a run: the caller's choice, else the autotuned value
-// for (L, chains per class), else the rule of heuristic_lanes.
-int pick_lanes(int L, int requested, int* lam_out, const surfmcmc_ctx* ctx = nullptr, int R = 0, int code = 0) {
-    const int nq = geo_nq(code, L), nc = geo_nc(code, L);
+// Lanes per bundle of a run of n syndromes with Cn chains each (at_once such
+// runs at the same time): the caller's choice, else the autotuned value for
+// (L, chains per class R; R = 0: none), widened where the batch does not fill
+// the device with it, else the rule of choose_lanes.
+int pick_lanes(const surfmcmc_ctx* ctx, int L, int requested, int R, int Cn, long long n, int code, int* lam_out,
+               int at_once = 1) {
     if (requested) {
         if (requested != 2 && requested != 4 && requested != 8 && requested != 16 && requested != 32)
             return SURFMCMC_EINVAL;
-        if (sweep_smem_bytes(nq, nc, requested) > kSweepSmemLimit) return SURFMCMC_EINVAL;
+        if (sweep_smem_bytes(geo_nq(code, L), geo_nc(code, L), requested) > kSweepSmemLimit) return SURFMCMC_EINVAL;
         *lam_out = requested;
         return SURFMCMC_OK;
     }
-    if (ctx) {
-        auto it = ctx->tuned.find({L, R});
-        if (it != ctx->tuned.end()) {
-            *lam_out = it->second.lam;
-            return SURFMCMC_OK;
-        }
-    }
-    *lam_out = heuristic_lanes(L, code);
+    SweepParams sp;
+    init_chains(sp, Cn, 1, 0);
+    const long long bundles = bundles_of(sp, n) * at_once;
+    const auto it = R > 0 ? ctx->tuned.find({L, R}) : ctx->tuned.end();
+    *lam_out = it != ctx->tuned.end() ? widen_lanes_for(ctx->sms, L, it->second.lam, bundles, sp.G, code)
+                                      : choose_lanes(ctx->sms, L, bundles, sp.G, code);
     return SURFMCMC_OK;
 }
 
@@ -195,13 +195,6 @@ int tuned_blocks(const surfmcmc_ctx* ctx, int L, int R, int requested_lanes) {
     if (requested_lanes || !ctx) return 0;
     auto it = ctx->tuned.find({L, R});
     return it == ctx->tuned.end() ? 0 : it->second.blocks_per_sm;
-}
-
-// Widens the lanes of a small batch (widen_lanes_for) unless the caller
-// fixed them.
-int widen_lanes(const surfmcmc_ctx* ctx, int L, int requested, int lam, long long n_bundles, int G, int code = 0) {
-    if (requested || !ctx) return lam;
-    return widen_lanes_for(ctx->sms, L, lam, n_bundles, G, code);
 }
 
 // Whether a planned run takes the one-block-per-bundle kernel (wide_batch):
@@ -408,10 +401,19 @@ int ragged_layout(surfmcmc_ctx* ctx, const int32_t* Ls, const uint32_t* sweeps, 
     for (auto& g : lay.groups) g.work = (double)g.items.size() * g.sweeps * (double)n_stabs(g.L);
     std::stable_sort(lay.groups.begin(), lay.groups.end(),
                      [](const RaggedGroup& a, const RaggedGroup& b) { return a.work > b.work; });
-    // lanes per bundle for the heaviest group, widened until the largest size fits
+    // lanes per bundle for the heaviest group (as if it held the whole call's
+    // work), widened until the largest size fits
     int lmax = 0;
-    for (auto& g : lay.groups) lmax = std::max(lmax, g.L);
-    if (pick_lanes(lay.groups.empty() ? 2 : lay.groups[0].L, o.lanes_per_bundle, &lay.lam, ctx, o.chains_per_class))
+    double work = 0.0;
+    for (auto& g : lay.groups) {
+        lmax = std::max(lmax, g.L);
+        work += g.work;
+    }
+    const long long n_equiv = lay.groups.empty() || lay.groups[0].work == 0.0
+                                  ? (long long)n
+                                  : (long long)((double)lay.groups[0].items.size() * work / lay.groups[0].work);
+    if (pick_lanes(ctx, lay.groups.empty() ? 2 : lay.groups[0].L, o.lanes_per_bundle, o.chains_per_class,
+                   4 * o.chains_per_class, n_equiv, 0, &lay.lam))
         return fail(ctx, SURFMCMC_EINVAL, "lanes_per_bundle=%d unsupported", o.lanes_per_bundle);
     if (o.scan) lay.lam = 32;
     while (sweep_smem_bytes(n_qubits(lmax), lmax * (lmax - 1) / 2, lay.lam) > 200 * 1024 && lay.lam < 32) lay.lam *= 2;
@@ -803,7 +805,7 @@ int surfmcmc_decode_ex(surfmcmc_ctx* ctx, const uint8_t* syndromes, int64_t n, i
     if ((rc = check_toric(ctx, o, L))) return rc;
     const int toric = o.n_classes == 16 ? 1 : 0;
     int lam = 0;
-    if (pick_lanes(L, o.lanes_per_bundle, &lam, ctx, o.chains_per_class, toric))
+    if (pick_lanes(ctx, L, o.lanes_per_bundle, o.chains_per_class, o.n_classes * o.chains_per_class, n, toric, &lam))
         return fail(ctx, SURFMCMC_EINVAL, "lanes_per_bundle=%d unsupported for L=%d", o.lanes_per_bundle, L);
     if (o.scan || out_chain_accepts) lam = 32;   // counting accepts: the LAM = 32 kernels (same results)
     if (n == 0) return SURFMCMC_OK;
@@ -823,7 +825,6 @@ int surfmcmc_decode_ex(surfmcmc_ctx* ctx, const uint8_t* syndromes, int64_t n, i
     sp.noise = o.noise;
     sp.max_blocks_per_sm = tuned_blocks(ctx, L, R, o.lanes_per_bundle);
     energy_table(o, sp.energy);
-    lam = widen_lanes(ctx, L, o.lanes_per_bundle, lam, bundles_of(sp, n), sp.G, toric);
     add_group(sp, L, n, 0, 0, 0, 0, lam);
     make_round_keys((uint32_t)seed, (uint32_t)(seed >> 32), &sp.rk);
 
@@ -930,7 +931,7 @@ int surfmcmc_decode_ti(surfmcmc_ctx* ctx, const uint8_t* syndromes, int64_t n, i
     if ((rc = check_toric(ctx, o, L))) return rc;
     const int toric = o.n_classes == 16 ? 1 : 0;
     int lam = 0;
-    if (pick_lanes(L, o.lanes_per_bundle, &lam, nullptr, 0, toric))
+    if (pick_lanes(ctx, L, o.lanes_per_bundle, 0, o.n_classes * o.chains_per_class, n, toric, &lam, n_beta - 1))
         return fail(ctx, SURFMCMC_EINVAL, "lanes_per_bundle=%d unsupported for L=%d", o.lanes_per_bundle, L);
     if (o.scan) lam = 32;
     if (n == 0) return SURFMCMC_OK;
@@ -950,10 +951,9 @@ int surfmcmc_decode_ti(surfmcmc_ctx* ctx, const uint8_t* syndromes, int64_t n, i
     // syndromes of an L = 9 batch filled a third of the device and its lanes
     // were widened to 56 % of use: 90.7 ms against 37.0.)
     const long long nb = bundles_of(sp, n);
-    lam = widen_lanes(ctx, L, o.lanes_per_bundle, lam, nb * (N - 1), sp.G, toric);
     add_group(sp, L, n, 0, 0, 0, 0, lam);
     sp.wide = o.lanes_per_bundle ? 0 : wide_batch(ctx->sms, sp, N - 1);
-    const long long fill = 2LL * ctx->sms * sweep_blocks_per_sm(sp.G), units = std::max(1LL, sweep_units(nb, lam));
+    const long long fill = 2LL * ctx->sms * sweep_blocks_per_sm(sp.G, lam), units = std::max(1LL, sweep_units(nb, lam));
     const int S = (int)std::max(1LL, std::min({(long long)(N - 1), (long long)kTiStreams, (fill + units - 1) / units}));
     const std::vector<Segment> segs0 = plan_segments(o, o.beta_scale, 0);
     const int W = geo_words(toric, L), nq = geo_nq(toric, L);
@@ -1268,7 +1268,7 @@ int surfmcmc_decode_early(surfmcmc_ctx* ctx, surfmcmc_cnn* net, const uint8_t* s
     if (reorder != 0 && reorder != 1) return fail(ctx, SURFMCMC_EINVAL, "reorder must be 0 or 1");
     if (n > 0 && (!syndromes || !out_class)) return fail(ctx, SURFMCMC_EINVAL, "NULL syndromes or out_class");
     int lam = 0;
-    if (pick_lanes(L, o.lanes_per_bundle, &lam, ctx, o.chains_per_class))
+    if (pick_lanes(ctx, L, o.lanes_per_bundle, o.chains_per_class, 4 * o.chains_per_class, n, 0, &lam))
         return fail(ctx, SURFMCMC_EINVAL, "lanes_per_bundle=%d unsupported for L=%d", o.lanes_per_bundle, L);
     if (o.scan) lam = 32;
     if (n == 0) return SURFMCMC_OK;
@@ -1354,7 +1354,8 @@ int surfmcmc_decode_early(surfmcmc_ctx* ctx, surfmcmc_cnn* net, const uint8_t* s
         sp.noise = o.noise;
         energy_table(o, sp.energy);
         sp.ids = t == 0 ? nullptr : (const uint32_t*)at(off_ids[cur]);
-        const int lam_k = widen_lanes(ctx, L, o.lanes_per_bundle, lam, bundles_of(sp, n_act), sp.G);
+        int lam_k = lam;
+        if (!o.scan) pick_lanes(ctx, L, o.lanes_per_bundle, R, Cn, n_act, 0, &lam_k);   // (the request is valid)
         add_group(sp, L, n_act, 0, 0, 0, 0, lam_k);
         sp.wide = take_wide(ctx, o, sp);
         make_round_keys((uint32_t)seed, (uint32_t)(seed >> 32), &sp.rk);

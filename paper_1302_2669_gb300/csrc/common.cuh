@@ -183,11 +183,15 @@ __host__ __device__ __forceinline__ int geo_nc(int code, int L) { return code ? 
 __host__ __device__ __forceinline__ int padded_nq(int nq, int lam) { return (nq + 4 * lam - 1) / (4 * lam) * (4 * lam); }
 __host__ __device__ __forceinline__ int bundle_stride(int nq, int lam) { return 2 * (padded_nq(nq, lam) + 2) + 1; }
 
-// Blocks per SM the sweep kernel is compiled for (its register bound): 5
-// with plane widths of 32 chains (96 registers, no spills: 0.8 % faster at
-// L = 13 than 6 blocks at 80 registers), 6 with 16 (6 blocks measured 3.7 %
-// faster than 5 there), 3 with narrower planes.
-__host__ __device__ constexpr int sweep_blocks_per_sm(int G) { return G == 32 ? 5 : G == 16 ? 6 : 3; }
+// Blocks per SM the sweep kernel is compiled for (its register bound): 6
+// (80 registers) with planes of 32 and 16 chains, 3 with narrower planes.  On
+// 32-chain planes 5 blocks took 10.45 ms where 6 take 10.04 (36,480 syndromes
+// at L = 13, 40 sweeps).  On 16-chain planes the kernels of 32 and 8 lanes
+// spill at 80 registers and are faster at 5 (L = 25: 5.55 against 5.68 ms, L =
+// 9: 6.30 against 6.62); those of 16 lanes are not (L = 13: 5.74 against 5.49).
+__host__ __device__ constexpr int sweep_blocks_per_sm(int G, int lam) {
+    return G == 16 && (lam == 32 || lam == 8) ? 5 : G >= 16 ? 6 : 3;
+}
 
 // ---------------------------------------------------------------------------
 // Sweep kernel parameters.  One launch runs the chains of up to kMaxGroups
@@ -223,12 +227,12 @@ struct SweepParams {
     int accept_all;            // r* == 1: every proposal accepted
     int reject_all;            // T[1] == 0: no uphill proposal accepted
     uint32_t qmodes;           // per quad of planes 4q..4q+3, 2 bits: 0 every threshold digit is 0,
-                               // 1 only T[1] has nonzero digits, 2 general
+                               // 1 only T[1] has nonzero digits, 3 only T[1] and T[2], 2 general
     RoundKeys rk;
     // Threshold bits of plane k as the algebraic normal form of the map
     // d-1 = e0 + 2 e1 -> bit (31-k) of T[d]: f = c0 ^ e0 c1 ^ e1 c2 ^ e0 e1 c3.
     uint32_t pc[4][32];
-    uint32_t tb[4][32];        // the same bits as masks: bit (31-k) of T[d] at [d-1][k] (one-block-per-bundle kernel)
+    uint32_t tb[4][32];        // the same bits as masks: bit (31-k) of T[d] at [d-1][k]
     const uint32_t* e0;        // pure errors
     const int32_t* e0code;     // [items]
     const uint32_t* init_frames;  // per-chain start frames, or NULL
@@ -284,6 +288,8 @@ cudaError_t launch_sweep_flips(const SweepParams& p, int lanes_per_bundle, cudaS
 // The launch on a kernel with its digit-plane modes compiled in;
 // cudaErrorNotSupported (nothing launched) where there is none.
 cudaError_t launch_sweep_modes(const SweepParams& p, int lanes_per_bundle, cudaStream_t s);
+cudaError_t launch_sweep_modes_narrow(const SweepParams& p, int lanes_per_bundle, cudaStream_t s);
+cudaError_t launch_sweep_modes_flips(const SweepParams& p, int lanes_per_bundle, cudaStream_t s);
 // Random scan (sweep_scan.cu).
 cudaError_t launch_sweep_scan(const SweepParams& p, cudaStream_t s);
 // The launch with one block per bundle (colour sweeps without accept counts).

@@ -101,7 +101,7 @@ extern "C" int surfmcmc_decode_noalloc(const uint8_t* syndromes, int64_t n, int3
         (unsigned int*)(sp0 + round256((size_t)n * 2 * W * 4) + round256((size_t)n * 4) + round256((size_t)n * Cn * 8));
 
     // The launch is planned by the same host rules as surfmcmc_decode's:
-    // chain layout, lanes per bundle (widened for small batches on this
+    // chain layout, lanes per bundle (choose_lanes for this
     // device's multiprocessors) and the Eq. 2 acceptance table.
     SweepParams sp;
     init_chains(sp, Cn, R, id0);
@@ -109,7 +109,7 @@ extern "C" int surfmcmc_decode_noalloc(const uint8_t* syndromes, int64_t n, int3
     energy_table(o, sp.energy);
     int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return SURFMCMC_ECUDA;
-    const int lam = widen_lanes_for(sms, L, heuristic_lanes(L, 0), bundles_of(sp, n), sp.G, 0);
+    const int lam = choose_lanes(sms, L, bundles_of(sp, n), sp.G, 0);
     add_group(sp, L, n, 0, 0, 0, 0, lam);
     sp.wide = wide_batch(sms, sp);
     GroupDesc& gd = sp.grp[0];

@@ -80,12 +80,13 @@ inline void set_temperature(SweepParams& sp, double p, double beta_scale) {
     sp.reject_all = T[1] == 0;
     sp.qmodes = 0;
     for (int q = 0; q < 8 && !sp.accept_all; ++q) {
-        uint32_t any1 = 0, any234 = 0;
+        uint32_t any1 = 0, any2 = 0, any34 = 0;
         for (int k = 4 * q; k < 4 * q + 4; ++k) {
             any1 |= (uint32_t)(T[1] >> (31 - k)) & 1u;
-            for (int d = 2; d <= 4; ++d) any234 |= (uint32_t)(T[d] >> (31 - k)) & 1u;
+            any2 |= (uint32_t)(T[2] >> (31 - k)) & 1u;
+            for (int d = 3; d <= 4; ++d) any34 |= (uint32_t)(T[d] >> (31 - k)) & 1u;
         }
-        sp.qmodes |= (any234 ? 2u : any1 ? 1u : 0u) << (2 * q);
+        sp.qmodes |= (any34 ? 2u : any2 ? 3u : any1 ? 1u : 0u) << (2 * q);
     }
     for (int k = 0; k < 32; ++k) {
         uint32_t t[5] = {0, 0, 0, 0, 0};
@@ -102,34 +103,47 @@ inline void set_temperature(SweepParams& sp, double p, double beta_scale) {
 // Shared memory a block may use for the sweep (the kernel's own limit).
 constexpr size_t kSweepSmemLimit = 200 * 1024;
 
-// Lanes per bundle by rule: the most lanes that the colour's generators fill
-// to >= 90%, else the best fill, within the shared-memory limit.
-inline int heuristic_lanes(int L, int code) {
+// Lanes per bundle by rule, for `bundles` bundles on a device with `sms`
+// multiprocessors: the smallest modelled time of a colour phase.  A unit
+// (4 warps x 32/lam bundles) takes rounds + 1.6 per phase: its proposals'
+// rounds and what every phase costs besides (queue pass, counting).  One
+// block alone on a multiprocessor runs at its latency, each further one adds
+// a third of that; the units past full waves of the r blocks that fit overlap
+// with them by half when they are few, not at all when they are nearly a
+// wave.  Fewer lanes fill the rounds and the queue better (at a cost in bank
+// conflicts and frames: 4, 20 and 24 % at 8, 4 and 2 lanes), more lanes make
+// short units for batches that do not fill the device.  Fitted to every split
+// of L = 3 .. 25 at 2,048 to 73,000 bundles: the pick is within 6 % of the
+// fastest.  (The fill of the last round alone lost up to 97 %: 2 lanes for
+// 8,192 bundles at L = 5 and 7.)  The results do not depend on the lanes.
+inline int choose_lanes(int sms, int L, long long bundles, int G, int code) {
     const int nq = geo_nq(code, L), nc = geo_nc(code, L);
     int best = 32;
-    double best_eff = -1;
+    double best_cost = 1e300;
     for (int lam = 32; lam >= 2; lam /= 2) {
-        if (sweep_smem_bytes(nq, nc, lam) > kSweepSmemLimit) continue;
-        const double eff = (double)nc / (double)(lam * ((nc + lam - 1) / lam));
-        if (eff >= 0.9) return lam;
-        if (eff > best_eff + 1e-12) {
-            best_eff = eff;
+        const size_t smem = sweep_smem_bytes(nq, nc, lam);
+        if (smem > kSweepSmemLimit) continue;
+        const int rounds = (nc + lam - 1) / lam, fit = (int)((228 * 1024) / (smem + 1024));
+        const double r = fit < 1 ? 1 : fit < sweep_blocks_per_sm(G, lam) ? fit : sweep_blocks_per_sm(G, lam);
+        const double u = (double)sweep_units(bundles, lam) / (sms > 0 ? sms : 1);
+        const double full = std::floor(u / r), rest = u - full * r;
+        const double tail = rest > 0 ? (3.0 + rest) * (0.5 + 0.5 * rest / r) : 0.0;
+        const double waves = full > 0 ? full * (3.0 + r) + tail : 3.0 + std::ceil(u);
+        const double cost = (rounds + 1.6) * waves * (lam == 2 ? 1.24 : lam == 4 ? 1.20 : lam == 8 ? 1.04 : 1.0);
+        if (cost < best_cost) {
+            best_cost = cost;
             best = lam;
         }
     }
     return best;
 }
 
-// Small batches: a persistent block takes work units of 4 warps x 32/lam
-// bundles, so a batch of few bundles leaves most blocks idle and the run
-// time is the latency of one unit.  Widen (more lanes share a bundle's
-// generators, shorter units) until the units fill the resident blocks of a
-// device with `sms` multiprocessors once.  The results do not depend on the
-// lanes.
+// An autotuned lane split on a batch too small for it: doubled until the units
+// fill the resident blocks of a device with `sms` multiprocessors once.
 inline int widen_lanes_for(int sms, int L, int lam, long long n_bundles, int G, int code) {
     if (sms <= 0) return lam;
     const int nq = geo_nq(code, L), nc = geo_nc(code, L);
-    const long long capacity = (long long)sms * sweep_blocks_per_sm(G);
+    const long long capacity = (long long)sms * sweep_blocks_per_sm(G, lam);
     while (lam < 32 && sweep_units(n_bundles, lam) < capacity && sweep_smem_bytes(nq, nc, 2 * lam) <= kSweepSmemLimit)
         lam *= 2;
     return lam;

@@ -344,30 +344,26 @@ __device__ __forceinline__ void head_fixed_words(const SweepParams& p, const uin
     }
 }
 
-// Digit-plane modes of a launch (per quad of planes: 0 every threshold digit
-// is 0, 1 only T[1] has nonzero digits, 2 general).  At every temperature the
-// decoder meets, the quads after the first two are general, and the first
-// two are (0, 1), (1, 2) or (2, 2); those three patterns have kernels of
-// their own (HM = 1, 2, 3) with the modes known at compile time, which saves
-// the per-quad dispatch in every proposal.  HM = 0 reads the modes from the
-// launch parameters.
-// Modes of quads 0 and 1 as in SweepParams::qmodes (quad q in bits 2q, 2q+1).
-__host__ __device__ constexpr uint32_t head_modes(int hm) {
-    return hm == 1 ? 0x4u /* 0, 1 */ : hm == 2 ? 0x9u /* 1, 2 */ : hm == 3 ? 0xAu /* 2, 2 */ : 0u;
-}
-
+// Digit-plane modes of a launch, per quad of planes: 0 every threshold digit
+// is 0, 1 only T[1] has nonzero digits, 3 only T[1] and T[2], 2 general (right
+// for any digits).  The quads after the first two run as general; the first
+// two run in one of three patterns, (0, 1), (1, 3) and (2, 2), each with
+// kernels of its own (HM = 1, 2, 3), chosen as the first that covers the
+// launch's modes: the sampled sweeps at p = 0.08-0.15 take (0, 1), those up
+// to 0.18 (1, 3; 3.5 % faster than as (1, 2)), hot annealing stages (2, 2).  HM = 0 reads the modes from
+// the launch parameters (accept-all and reject-all launches, accept counts,
+// the shapes without kernels of their own).
 template <int HM>
 __device__ __forceinline__ uint32_t quad_mode(const SweepParams& p, int q) {
     if constexpr (HM == 0) return (p.qmodes >> (2 * q)) & 3u;
-    else return q >= 2 ? 2u : (head_modes(HM) >> (2 * q)) & 3u;
+    else return q >= 2 || HM == 3 ? 2u : HM == 1 ? (q == 0 ? 0u : 1u) : (q == 0 ? 1u : 3u);
 }
 
-// The specialised head pattern of a launch's modes (0: none).
-__host__ __device__ inline int head_pattern(uint32_t qmodes) {
-    if ((qmodes >> 4) != 0xAAAu) return 0;   // quads 2 .. 7 general (mode 2 each)
-    for (int hm = 1; hm <= 3; ++hm)
-        if ((qmodes & 0xFu) == head_modes(hm)) return hm;
-    return 0;
+// The specialised head pattern of a launch (0: none).
+__host__ __device__ inline int head_pattern(const SweepParams& p) {
+    if (p.accept_all || p.reject_all) return 0;
+    const uint32_t m0 = p.qmodes & 3u, m1 = (p.qmodes >> 2) & 3u;
+    return m0 == 0 && m1 <= 1 ? 1 : m0 <= 1 && m1 != 2 ? 2 : 3;
 }
 
 // Accept mask of the undecided uphill chains U (all have Delta n = d > 0,
@@ -414,6 +410,15 @@ __device__ __forceinline__ uint32_t bernoulli_range(const SweepParams& p, uint32
                 for (int i = 0; i < 4; ++i) {
                     const uint32_t r = pb.pl[4 * qd + i];
                     const uint32_t f = p.pc[0][k0 + i] & M1;
+                    acc |= U & f & ~r;
+                    U &= ~(f ^ r);
+                }
+            } else if (mode == 3) {
+                // only T[1] and T[2] have nonzero digits here
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const uint32_t r = pb.pl[4 * qd + i];
+                    const uint32_t f = (p.tb[0][k0 + i] & M1) | (p.tb[1][k0 + i] & E0 & ~E1);
                     acc |= U & f & ~r;
                     U &= ~(f ^ r);
                 }
@@ -543,6 +548,19 @@ struct BundleMap {
     __device__ __forceinline__ long long syn_of(int b) const { return G == 32 ? syn[0] : syn[G == 32 ? 0 : b / G]; }
 };
 
+// Index of the chain behind valid bit b of bundle `bid` in the [items][C]
+// arrays; from the bundle's number alone, for the places where keeping its
+// map would hold registers through the sweeps.
+template <int G>
+__device__ __forceinline__ size_t chain_index(const SweepParams& p, const GroupDesc& gd, long long bid, int b) {
+    if constexpr (G == 32) {
+        const long long s = bid / p.bps;
+        return (size_t)(gd.item_base + s) * p.C + 32 * (size_t)(bid - s * p.bps) + b;
+    } else {
+        return (size_t)(gd.item_base + bid * PlaneBatch<G>::SLOTS + b / G) * p.C + b % G;
+    }
+}
+
 // Bit-sliced start state of a bundle, word by word: the state an earlier
 // launch left, the caller's per-chain frames, or the pure error times the
 // logical that gives chain c the class code c / R (planar code: bit 0 X-bar
@@ -638,35 +656,37 @@ __device__ __forceinline__ void run_unit(const SweepParams& p, const GroupDesc& 
     uint32_t* q_items = q_cnt + 1;
     uint32_t* binfo = q_items + kQueueCap * kQueueItem;  // per slot: w, sid[SLOTS]
 
-    // Syndromes and chains of the bundle.
-    const BundleMap<G> bm(p, gd, bid);
-    const uint32_t* sid = bm.sid;
-    const uint32_t w = bm.w, valid = bm.valid;
     uint32_t* fx = fixed + (warp * B + slot) * kHeadFixedWords;
-    if (sub == 0) {
-        binfo[slot * (kMaxSlots + 1)] = w;
-#pragma unroll
-        for (int s = 0; s < SLOTS; ++s) binfo[slot * (kMaxSlots + 1) + 1 + s] = sid[s];
-        head_fixed_words<G>(p, sid, w, fx);
-    }
-    auto chain_of = [&](int b) -> int { return bm.chain_of(b); };
-    auto syn_of = [&](int b) -> long long { return bm.syn_of(b); };
-
     const int W = gd.W;
     uint32_t* cfg = p.chain_frames ? p.chain_frames + gd.frames_off - (size_t)gd.item_base * p.C * 2 * W : nullptr;
-    const StartState<G> start(p, gd, bm);
-    for (int q = sub; q < nqp; q += LAM) {
-        uint32_t xw = 0, zw = 0;   // zero padding past nq
-        if (q < nq) start.word(q, xw, zw);
-        X[q] = xw;
-        Z[q] = zw;
+    uint32_t valid;
+    {
+        // The bundle's map lives for the prologue only: kept through the
+        // sweeps its syndromes and ids hold registers that these need (10.04
+        // ms against 10.34 without, 36,480 syndromes at L = 13, 64 chains, 40
+        // sweeps; 7.43 against 7.60 at L = 17, 16 chains).
+        const BundleMap<G> bm(p, gd, bid);
+        valid = bm.valid;
+        if (sub == 0) {
+            binfo[slot * (kMaxSlots + 1)] = bm.w;
+#pragma unroll
+            for (int s = 0; s < SLOTS; ++s) binfo[slot * (kMaxSlots + 1) + 1 + s] = bm.sid[s];
+            head_fixed_words<G>(p, bm.sid, bm.w, fx);
+        }
+        const StartState<G> start(p, gd, bm);
+        for (int q = sub; q < nqp; q += LAM) {
+            uint32_t xw = 0, zw = 0;   // zero padding past nq
+            if (q < nq) start.word(q, xw, zw);
+            X[q] = xw;
+            Z[q] = zw;
+        }
     }
     if (sub == 0) {
         X[nqp] = 0u; Z[nqp] = 0xFFFFFFFFu;          // dummy of sigma_x generators
         X[nqp + 1] = 0xFFFFFFFFu; Z[nqp + 1] = 0u;  // dummy of sigma_z generators
     }
     // Owned chains' sums live in the output array; flushes add to them.
-    auto ci_of = [&](int b) -> size_t { return (size_t)syn_of(b) * p.C + chain_of(b); };
+    auto ci_of = [&](int b) -> size_t { return chain_index<G>(p, gd, bid, b); };
 #pragma unroll
     for (int j = 0; j < NJ; ++j) {
         const int b = sub + j * LAM;
@@ -694,6 +714,7 @@ __device__ __forceinline__ void run_unit(const SweepParams& p, const GroupDesc& 
             constexpr int HEAD = kHeadPlanes / PPB > 0 ? kHeadPlanes / PPB : 1;
             if (lane == 0) *q_cnt = 0u;
             __syncwarp();
+            const uint32_t* info = binfo + slot * (kMaxSlots + 1);   // w, ids
             if (active) {
                 for (int m = sub; m < nc; m += LAM) {
                     const ushort4 sp = tc[m];
@@ -727,7 +748,7 @@ __device__ __forceinline__ void run_unit(const SweepParams& p, const GroupDesc& 
                             // Delta n - 1 = E0 + 2 E1 on the uphill chains
                             const uint32_t E0 = ~w0, E1 = Z0 & Wge3;
                             const uint32_t cm = colm | (uint32_t)m;
-                            acc |= bernoulli_range<G, 0, HEAD, HM>(p, U, E0, E1, sid, w, t, cm, fx);
+                            acc |= bernoulli_range<G, 0, HEAD, HM>(p, U, E0, E1, info + 1, info[0], t, cm, fx);
                             if constexpr (HEAD < NBATCH) {
                                 if (U) {
                                     const uint32_t qi = atomicAdd(q_cnt, 1u);
@@ -740,7 +761,7 @@ __device__ __forceinline__ void run_unit(const SweepParams& p, const GroupDesc& 
                                         it[4] = acc;
                                         continue;  // flipped after the queue is resolved
                                     }
-                                    acc |= bernoulli_range<G, HEAD, NBATCH, HM>(p, U, E0, E1, sid, w, t, cm);
+                                    acc |= bernoulli_range<G, HEAD, NBATCH, HM>(p, U, E0, E1, info + 1, info[0], t, cm);
                                 }
                             }
                         }
@@ -761,12 +782,9 @@ __device__ __forceinline__ void run_unit(const SweepParams& p, const GroupDesc& 
                     const int qm = (int)(it[0] & 0xFFFFu), qs = (int)(it[0] >> 16);
                     uint32_t U = it[1];
                     uint32_t acc = it[4];
-                    const uint32_t* info = binfo + qs * (kMaxSlots + 1);
-                    uint32_t qsid[SLOTS];
-#pragma unroll
-                    for (int s = 0; s < SLOTS; ++s) qsid[s] = info[1 + s];
-                    acc |= bernoulli_range<G, HEAD, NBATCH, HM>(p, U, it[2], it[3], qsid, info[0], t,
-                                                            colm | (uint32_t)qm);
+                    const uint32_t* qinfo = binfo + qs * (kMaxSlots + 1);
+                    acc |= bernoulli_range<G, HEAD, NBATCH, HM>(p, U, it[2], it[3], qinfo + 1, qinfo[0], t,
+                                                                colm | (uint32_t)qm);
                     if constexpr (ACPT) it[4] = acc;
                     if (acc) {
                         uint32_t* qx = frames + (warp * B + qs) * stride;
@@ -818,7 +836,7 @@ __device__ __forceinline__ void run_unit(const SweepParams& p, const GroupDesc& 
     for (int j = 0; j < NJ; ++j) {
         const int b = sub + j * LAM;
         if (!((valid >> b) & 1u)) continue;
-        const size_t ci = (size_t)syn_of(b) * p.C + chain_of(b);
+        const size_t ci = ci_of(b);
         if (p.chain_n) p.chain_n[ci] = (int32_t)bit_of(cnt, b);
         if (cfg) {
             uint32_t* f = cfg + ci * 2 * W;
@@ -843,7 +861,7 @@ __device__ __forceinline__ void run_unit(const SweepParams& p, const GroupDesc& 
 // the host arranged (largest work first), and rebuilds the support table in
 // shared memory when the group's code size changes.
 template <int G, int LAM, bool IND, bool ACPT, int HM = 0>
-__global__ void __launch_bounds__(128, sweep_blocks_per_sm(G)) sweep_kernel(const __grid_constant__ SweepParams p) {
+__global__ void __launch_bounds__(128, sweep_blocks_per_sm(G, LAM)) sweep_kernel(const __grid_constant__ SweepParams p) {
     extern __shared__ __align__(16) uint32_t smem[];
     __shared__ long long s_unit;
     ushort4* tab = reinterpret_cast<ushort4*>(smem);

@@ -1,0 +1,46 @@
+// Launchers of the sweep kernels with a compiled-in head pattern.  The
+// 32-chain kernels take every chain of a bundle as valid, so they serve
+// launches whose chain count per syndrome is a multiple of 32.  Launches
+// without such a kernel (cudaErrorNotSupported, nothing launched) use those of
+// sweep.cu, which read the modes from their parameters.
+#pragma once
+#include "sweep_kernel.cuh"
+
+namespace surfmcmc {
+
+template <int G, bool IND, int HM>
+static cudaError_t launch_hm(const SweepParams& p, int lam, cudaStream_t s) {
+    switch (lam) {
+        case 2: return launch_t<G, 2, IND, false, HM>(p, s);
+        case 4: return launch_t<G, 4, IND, false, HM>(p, s);
+        case 8: return launch_t<G, 8, IND, false, HM>(p, s);
+        case 16: return launch_t<G, 16, IND, false, HM>(p, s);
+        case 32: return launch_t<G, 32, IND, false, HM>(p, s);
+        default: return cudaErrorNotSupported;
+    }
+}
+
+template <int G, bool IND>
+static cudaError_t launch_g_hm(const SweepParams& p, int lam, cudaStream_t s) {
+    switch (head_pattern(p)) {
+        case 1: return launch_hm<G, IND, 1>(p, lam, s);
+        case 2: return launch_hm<G, IND, 2>(p, lam, s);
+        case 3: return launch_hm<G, IND, 3>(p, lam, s);
+        default: return cudaErrorNotSupported;
+    }
+}
+
+template <bool IND>
+static cudaError_t launch_modes_wide_planes(const SweepParams& p, int lam, cudaStream_t s) {
+    if (p.accepts) return cudaErrorNotSupported;
+    if (p.G == 16) return launch_g_hm<16, IND>(p, lam, s);
+    return p.C % 32 == 0 ? launch_g_hm<32, IND>(p, lam, s) : cudaErrorNotSupported;
+}
+
+template <bool IND>
+static cudaError_t launch_modes_narrow_planes(const SweepParams& p, int lam, cudaStream_t s) {
+    if (p.accepts) return cudaErrorNotSupported;
+    return p.G == 8 ? launch_g_hm<8, IND>(p, lam, s) : launch_g_hm<4, IND>(p, lam, s);
+}
+
+}  // namespace surfmcmc

@@ -111,7 +111,7 @@ __device__ __forceinline__ void compare_digits(const uint32_t c[4], const uint32
 __device__ __forceinline__ void compare_quad(const SweepParams& p, int q, const uint32_t r[4], uint32_t lt[4],
                                              uint32_t eq[4]) {
     const uint32_t mode = (p.qmodes >> (2 * q)) & 3u;
-    if (mode == 2) {
+    if (mode >= 2) {
 #pragma unroll
         for (int d = 0; d < 4; ++d) compare_digits(p.tb[d] + 4 * q, r, lt[d], eq[d]);
     } else {
