@@ -13,9 +13,13 @@
 // +-(1 - 1e-6), and log p_{a + 2b} = log P_x(a xor a0) + log P_z(b xor b0).
 //
 // Layouts: activations are NHWC bfloat16, [M][C] with M = n P^2 positions of
-// the maps zero-padded to P = L + 2 (syndrome-major, then row, then column):
-// every 3x3 tap is then a shift of the position index by dy P + dx, and the
-// epilogues keep the one-position border at zero.  Weights live as float32 master
+// the maps followed by one zero column and one zero row, P = L + 1
+// (syndrome-major, then row, then column): every 3x3 tap is then a shift of
+// the position index by dy P + dx, whose steps left of column 0 and above row
+// 0 land on the zero column of the row and the zero row of the map before
+// (before the first map: on the zero fill of the TMA loads), and the
+// epilogues keep the border at zero.  (A border on all four sides, P = L + 2,
+// is 11 % more positions at L = 17: 731 us for 8,192 syndromes against 665.)  Weights live as float32 master
 // copies in the flat order W[co][kh][kw][ci] then b[co], layer after layer;
 // every step packs them into bfloat16 GEMM operands.
 //
@@ -286,16 +290,19 @@ __device__ __forceinline__ bool epi_all(bool v, uint32_t id = 1) {
     return r != 0;
 }
 
-// Padded maps: P = L + 2; interior positions are the L x L map, the rest is
-// the zero border.  Whether position rem = m mod P^2 inside its map is
-// interior:
+// Maps of P x P positions, P = L + 1; interior positions are the L x L map,
+// row L and column L the zero border.  Whether position rem = m mod P^2 inside
+// its map is interior:
+__host__ __device__ __forceinline__ constexpr int map_pitch(int L) { return L + 1; }
 __device__ __forceinline__ bool interior_rem(int rem, int L) {
-    const int P = L + 2, y = rem / P, x = rem - y * P;
-    return y >= 1 && y <= L && x >= 1 && x <= L;
+    const int P = map_pitch(L), y = rem / P, x = rem - y * P;
+    return y < L && x < L;
 }
 
 // Position shift of tap t = 3 kh + kw: (kh - 1) P + (kw - 1).
-__device__ __forceinline__ int tap_shift(int t, int L) { return (t / 3 - 1) * (L + 2) + (t % 3 - 1); }
+__device__ __forceinline__ int tap_shift(int t, int L) { return (t / 3 - 1) * map_pitch(L) + (t % 3 - 1); }
+// Largest shift.
+__host__ __device__ __forceinline__ constexpr int tap_reach(int L) { return map_pitch(L) + 1; }
 
 // 64 consecutive f32 columns of this warp's 32 tensor-memory lanes, one
 // load and one wait.
@@ -360,9 +367,9 @@ constexpr int kC1StripStage = 1024;             // one tile's input strip
 constexpr int kC1Threads = 14 * 32;             // TMA warp, MMA warp, 2 x 4 accumulator warps, 4 operand warps
 
 // 16-byte rows (4 positions) of the input strip of a 128-position tile: the
-// taps reach P + 1 = L + 3 positions either way and the strip starts up to 3
+// taps reach P + 1 positions either way and the strip starts up to 3
 // positions before the first one it needs (row-aligned).
-__host__ __device__ constexpr int c1_strip_rows(int L) { return (128 + 2 * (L + 3) + 3 + 3) / 4; }
+__host__ __device__ constexpr int c1_strip_rows(int L) { return (128 + 2 * tap_reach(L) + 3 + 3) / 4; }
 static_assert(c1_strip_rows(SURFMCMC_MAX_L) * 16 <= kC1StripStage, "input strip");
 constexpr size_t kC1Smem = 4 * (size_t)kOutTile + kC1S * kC1Stage + 64 * kC1KP * 2 + kC1S * kC1StripStage + 1024;
 
@@ -397,7 +404,7 @@ __global__ void __launch_bounds__(kC1Threads, 1) conv1_kernel(const __grid_const
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const long long M = a.M;
-    const int L = a.L, P1 = L + 3;
+    const int L = a.L, P1 = tap_reach(L);
     const long long n_tiles = (M + 127) / 128;
 
     for (int idx = tid; idx < NP * KGS; idx += kC1Threads) {
@@ -468,7 +475,7 @@ __global__ void __launch_bounds__(kC1Threads, 1) conv1_kernel(const __grid_const
     } else if (warp >= 10) {
         // operand rows: thread r builds row r of every tile
         const int r = 32 * (warp - 10) + lane;
-        const int PP = (L + 2) * (L + 2);
+        const int PP = map_pitch(L) * map_pitch(L);
         int sh[9];
 #pragma unroll
         for (int t = 0; t < 9; ++t) sh[t] = tap_shift(t, L);
@@ -558,10 +565,10 @@ struct ConvTmaArgs {
 };
 
 // Rows of the halo tile of 128 output positions: the taps shift by up to
-// P + 1 = L + 3 rows either way; rounded up to whole 8-row swizzle atoms so
+// P + 1 rows either way; rounded up to whole 8-row swizzle atoms so
 // that every stage starts on a 1024-byte boundary.  At most 200 (L = 31),
 // inside the 256-row limit of a TMA box.
-__host__ __device__ constexpr int halo_tile_rows(int L) { return (128 + 2 * (L + 3) + 7) / 8 * 8; }
+__host__ __device__ constexpr int halo_tile_rows(int L) { return (128 + 2 * tap_reach(L) + 7) / 8 * 8; }
 constexpr int kHaloRowsMax = halo_tile_rows(SURFMCMC_MAX_L);
 constexpr int kTmaStage = kHaloRowsMax * 128;   // stage stride in bytes
 static_assert(kHaloRowsMax <= 256 && kTmaStage % 1024 == 0, "halo tile");
@@ -609,7 +616,7 @@ __global__ void __launch_bounds__(kTmaThreads, 1) conv_tma_kernel(const __grid_c
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const long long M = a.M;
-    const int L = a.L, P1 = L + 3;
+    const int L = a.L, P1 = tap_reach(L);
     const long long n_tiles = (M + 127) / 128;
 
     for (int idx = tid; idx < NP * KG; idx += kTmaThreads) {
@@ -693,7 +700,7 @@ __global__ void __launch_bounds__(kTmaThreads, 1) conv_tma_kernel(const __grid_c
         const int quarter = warp & 3;
         const int row = 32 * quarter + lane;
         const bool elected = warp == 2 && lane == 0;
-        const int PP = (L + 2) * (L + 2);
+        const int PP = map_pitch(L) * map_pitch(L);
         float bias[EPI == kEpiRelu ? NP : 1];
 #pragma unroll
         for (int j = 0; j < (EPI == kEpiRelu ? NP : 1); ++j) bias[j] = EPI == kEpiRelu ? __ldg(a.bias + j) : 0.0f;
@@ -803,7 +810,7 @@ struct WgradArgs {
 };
 
 constexpr int kWgS = 4;                          // pipeline depth
-__host__ __device__ constexpr int wg_halo_rows(int L) { return (64 + 2 * (L + 3) + 7) / 8 * 8; }
+__host__ __device__ constexpr int wg_halo_rows(int L) { return (64 + 2 * tap_reach(L) + 7) / 8 * 8; }
 constexpr int kWgXStage = wg_halo_rows(SURFMCMC_MAX_L) * 128;   // 17 KB at L = 31
 constexpr int kWgDStage = 64 * 128;
 constexpr int kWgStage = kWgXStage + kWgDStage;
@@ -828,7 +835,7 @@ __global__ void __launch_bounds__(kWgTmaThreads, 1) wgrad_kernel(const __grid_co
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const long long M = a.M;
-    const int L = a.L, P1 = L + 3;
+    const int L = a.L, P1 = tap_reach(L);
     const long long n_chunks = (M + 63) / 64;
     const long long c_begin = n_chunks * blockIdx.x / gridDim.x, c_end = n_chunks * (blockIdx.x + 1) / gridDim.x;
 
@@ -985,7 +992,7 @@ __global__ void __launch_bounds__(kW0Threads, 1) wgrad0_kernel(const __grid_cons
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const long long M = a.M;
-    const int L = a.L, P1 = L + 3;
+    const int L = a.L, P1 = tap_reach(L);
     const long long n_chunks = (M + 127) / 128;
     const long long c_begin = n_chunks * blockIdx.x / gridDim.x, c_end = n_chunks * (blockIdx.x + 1) / gridDim.x;
 
@@ -1133,18 +1140,18 @@ __global__ void __launch_bounds__(256) wgrad_reduce_kernel(const float* partial,
 // CUDA-core kernels
 // ---------------------------------------------------------------------------
 
-// Syndromes [n][2L(L-1)] -> padded input maps [n P^2][2]: channel 0 the
-// sigma_x generators ((L-1) x L, last row zero), channel 1 the sigma_z
-// generators (L x (L-1), last column zero); map (y, x) at padded (y+1, x+1).
+// Syndromes [n][2L(L-1)] -> input maps [n P^2][2]: channel 0 the sigma_x
+// generators ((L-1) x L, last row zero), channel 1 the sigma_z generators
+// (L x (L-1), last column zero).
 __global__ void input_maps_kernel(const uint8_t* syn, long long n, int L, bf16* x0) {
     const long long m = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const int P = L + 2;
+    const int P = map_pitch(L);
     const long long PP = (long long)P * P;
     if (m >= n * PP) return;
     const long long item = m / PP;
-    const int rem = (int)(m - item * PP), y = rem / P - 1, x = rem - (rem / P) * P - 1;
+    const int rem = (int)(m - item * PP), y = rem / P, x = rem - y * P;
     float c0 = 0.0f, c1 = 0.0f;
-    if (y >= 0 && y < L && x >= 0 && x < L) {
+    if (y < L && x < L) {
         const uint8_t* s = syn + item * 2 * L * (L - 1);
         c0 = y < L - 1 ? (float)(s[y * L + x] & 1) : 0.0f;
         c1 = x < L - 1 ? (float)(s[L * (L - 1) + y * (L - 1) + x] & 1) : 0.0f;
@@ -1230,8 +1237,8 @@ __global__ void __launch_bounds__(256, 4) readout_kernel(const bf16* w5, const f
     const long long item = (long long)blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (item >= n) return;
-    const int m = (L - 1) / 2, P = L + 2;
-    const long long base = item * P * P + P + 1;   // map (0, 0)
+    const int m = (L - 1) / 2, P = map_pitch(L);
+    const long long base = item * P * P;   // map (0, 0)
     const uint32_t* a = reinterpret_cast<const uint32_t*>(a4) + lane;   // 32 words per position
     float sa = 0.0f, sb = 0.0f;
     for (int i = 0; i < L; i += kReadK) {
@@ -1241,7 +1248,7 @@ __global__ void __launch_bounds__(256, 4) readout_kernel(const bf16* w5, const f
 #pragma unroll
         for (int r = 0; r < kReadK + 2; ++r) {
             const int y = i - 1 + r;             // <= L: the bottom (right) border at most
-            const bool ok = y <= L;
+            const bool ok = y >= 0 && y <= L;    // above row 0 (left of column 0): zero
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
                 la[r][c] = ok ? __ldg(a + (base + (long long)y * P + (m - 1 + c)) * 32) : 0u;
@@ -1361,7 +1368,7 @@ __global__ void conv5_dgrad_kernel(const bf16* w5, const float* dz5, const bf16*
     if (i >= n * NB * 8) return;
     const long long item = i / (NB * 8);
     const int j = (int)(i / 8 - item * NB), cg = (int)(i & 7) * 8;
-    const int m = (L - 1) / 2, P = L + 2;
+    const int m = (L - 1) / 2, P = map_pitch(L);
     int y, x;
     if (j < 3 * L) {
         y = m - 1 + j / L;
@@ -1372,10 +1379,11 @@ __global__ void conv5_dgrad_kernel(const bf16* w5, const float* dz5, const bf16*
         if (y >= m - 1 && y <= m + 1) return;   // in the row band
     }
     if (y < 0 || y >= L || x < 0 || x >= L) return;
-    const long long q = item * P * P + (long long)(y + 1) * P + (x + 1);
+    const long long q = item * P * P + (long long)y * P + x;
     float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     bool any = false;
     for (int t = 0; t < 9; ++t) {
+        if (y - (t / 3 - 1) < 0 || x - (t % 3 - 1) < 0) continue;   // outside the map: zero
         const float2 d = *reinterpret_cast<const float2*>(dz5 + (q - tap_shift(t, L)) * 2);
         if (d.x == 0.0f && d.y == 0.0f) continue;
         any = true;
@@ -1403,22 +1411,22 @@ __global__ void conv5_dgrad_kernel(const bf16* w5, const float* dz5, const bf16*
 // a4[p + shift(tap)][ci] over the item's positions p, Sb[item][co] = sum_p
 // dz5[p][co].  dz5 is nonzero only on channel 0 of the middle column and
 // channel 1 of the middle row, so the sums run over those lines, row by row
-// (column by column).  The neighbours of a map position lie in the item's
-// padded frame.
+// (column by column).
 __global__ void conv5_wgrad_item_kernel(const float* dz5, const bf16* a4, int L, float* S, float* Sb) {
     const long long item = blockIdx.x;
     const int t = threadIdx.x >> 6, ci = threadIdx.x & 63;
-    const int P = L + 2, PP = P * P, sh = tap_shift(t, L), m = (L - 1) / 2;
+    const int P = map_pitch(L), PP = P * P, dy = t / 3 - 1, dx = t % 3 - 1, m = (L - 1) / 2;
     const float* d = dz5 + item * PP * 2;
     const bf16* a = a4 + item * (long long)PP * 64;
     float acc0 = 0.0f, acc1 = 0.0f, b0 = 0.0f, b1 = 0.0f;
     for (int i = 0; i < L; ++i) {
-        const int pa = (i + 1) * P + m + 1, pb = (m + 1) * P + i + 1;
+        const int pa = i * P + m, pb = m * P + i;
         const float d0 = d[2 * pa], d1 = d[2 * pb + 1];
         b0 += d0;
         b1 += d1;
-        acc0 += d0 * __bfloat162float(a[(pa + sh) * 64 + ci]);
-        acc1 += d1 * __bfloat162float(a[(pb + sh) * 64 + ci]);
+        // (above row 0, left of column 0: zero; m >= 1, so the other index is inside)
+        if (i + dy >= 0) acc0 += d0 * __bfloat162float(a[((i + dy) * P + m + dx) * 64 + ci]);
+        if (i + dx >= 0) acc1 += d1 * __bfloat162float(a[((m + dy) * P + i + dx) * 64 + ci]);
     }
     S[(item * 2 + 0) * 576 + threadIdx.x] = acc0;
     S[(item * 2 + 1) * 576 + threadIdx.x] = acc1;
@@ -1849,7 +1857,7 @@ int surfmcmc_cnn_create(surfmcmc_ctx* ctx, int32_t L, int64_t max_batch, surfmcm
     net->ctx = ctx;
     net->device = ctx_device(ctx);
     net->L = L;
-    net->P = L + 2;
+    net->P = map_pitch(L);
     net->max_batch = max_batch;
     NetGuard g(net->device);
     cudaError_t e = cudaDeviceGetAttribute(&net->sms, cudaDevAttrMultiProcessorCount, net->device);
