@@ -19,7 +19,8 @@
 //
 // Measured (GB300, L = 9, 4,096 syndromes x 16 chains, 200 sweeps): 24.5 ms on
 // the bit-sliced frames this replaced (8 loads and 4 atomics per step on
-// random banks, the energy of each qubit by selects), 10.9 ms here.
+// random banks, the energy of each qubit by selects), 10.1 ms here (10.9 before
+// the planar code took its two middle bits together).
 #include <algorithm>
 
 #include "sweep_kernel.cuh"
@@ -111,6 +112,9 @@ __device__ __forceinline__ uint2 scan_move(const SweepParams& p, int type, int s
     return make_uint2(always ? 0u : (uint32_t)p.T[dn], (uint32_t)(2 * dn) | (always ? 1u : 0u));
 }
 
+// v >> (s mod 32)
+__device__ __forceinline__ uint32_t shr(uint32_t v, uint32_t s) { return v >> (s & 31u); }
+
 // Words 0 and 1 of Philox4x32-10 for the counters (id, chain, t, step) of one
 // sweep: the rounds' parts that do not depend on the step.
 struct ScanPhilox {
@@ -134,7 +138,7 @@ struct ScanPhilox {
     }
 };
 
-template <int G>
+template <int G, bool TORIC>
 __global__ void __launch_bounds__(32 * kScanWarps) scan_kernel(const __grid_constant__ SweepParams p) {
     extern __shared__ __align__(16) uint32_t smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -213,7 +217,8 @@ __global__ void __launch_bounds__(32 * kScanWarps) scan_kernel(const __grid_cons
             for (int k = 0; k < U; ++k) {
                 const uint32_t own = base + ((int)tbl[k] < 0 ? plane : 0u), oth = base + ((int)tbl[k] < 0 ? 0u : plane);
                 const uint32_t rm = e[k] & 0x1F80u, ru = (e[k] >> 6) & 0x1F80u, rd = (e[k] >> 12) & 0x1F80u;
-                const uint32_t bl = e[k] & 31u, br = (e[k] >> 25) & 31u, bu = e[k] & 32u ? br : bl;
+                const uint32_t bl = e[k], br = e[k] >> 25;   // (shifts take the low 5 bits)
+                const uint32_t bu = TORIC ? (e[k] & 32u ? br : bl) : bl + ((e[k] >> 5) & 1u);
                 auto ld = [](uint32_t a) {
                     uint32_t v;
                     asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
@@ -224,19 +229,27 @@ __global__ void __launch_bounds__(32 * kScanWarps) scan_kernel(const __grid_cons
                 };
                 const uint32_t om = ld(own + rm), ou = ld(own + ru), od = ld(own + rd);
                 const uint32_t tm = ld(oth + rm), tu = ld(oth + ru), td = ld(oth + rd);
-                uint32_t idx = (om >> bl) & 1u;
-                idx |= ((om >> br) & 1u) << 1;
-                idx |= ((ou >> bu) & 1u) << 2;
-                idx |= ((od >> bu) & 1u) << 3;
-                idx |= ((tm >> bl) & 1u) << 4;
-                idx |= ((tm >> br) & 1u) << 5;
-                idx |= ((tu >> bu) & 1u) << 6;
-                idx |= ((td >> bu) & 1u) << 7;
+                // own l, r, u, d in bits 0-3, other l, r, u, d in bits 4-7; the
+                // planar code's r is the bit after l
+                uint32_t o, x;
+                if (TORIC) {
+                    o = (shr(om, bl) & 1u) + 2u * (shr(om, br) & 1u);
+                    x = (shr(tm, bl) & 1u) + 2u * (shr(tm, br) & 1u);
+                } else {
+                    o = shr(om, bl) & 3u;
+                    x = shr(tm, bl) & 3u;
+                }
+                o += 4u * (shr(ou, bu) & 1u);
+                x += 4u * (shr(tu, bu) & 1u);
+                o += 8u * (shr(od, bu) & 1u);
+                x += 8u * (shr(td, bu) & 1u);
+                const uint32_t idx = o + 16u * x;
                 const uint2 mv = moves[(tbl[k] & 0x7FFFFFFFu) + idx];
                 if (u[k] < mv.x || (mv.y & 1u)) {
-                    st(own + rm, om ^ (1u << bl) ^ (1u << br));
-                    st(own + ru, ou ^ (1u << bu));
-                    st(own + rd, od ^ (1u << bu));
+                    const uint32_t up = 1u << (bu & 31u);
+                    st(own + rm, om ^ (TORIC ? 1u << (bl & 31u) ^ 1u << (br & 31u) : 3u << (bl & 31u)));
+                    st(own + ru, ou ^ up);
+                    st(own + rd, od ^ up);
                     n += (int)mv.y >> 1;
                     ++accepted;
                 }
@@ -280,8 +293,8 @@ __global__ void __launch_bounds__(32 * kScanWarps) scan_kernel(const __grid_cons
     }
 }
 
-template <int G>
-cudaError_t launch_scan_g(const SweepParams& p, cudaStream_t s) {
+template <int G, bool TORIC>
+cudaError_t launch_scan_t(const SweepParams& p, cudaStream_t s) {
     long long blocks = 0;
     size_t smem = 0;
     for (int g = 0; g < p.n_groups; ++g) {
@@ -292,10 +305,15 @@ cudaError_t launch_scan_g(const SweepParams& p, cudaStream_t s) {
     static SmemLimit limit;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess && smem > 48 * 1024) e = limit.ensure(scan_kernel<G>, dev, smem);
+    if (e == cudaSuccess && smem > 48 * 1024) e = limit.ensure(scan_kernel<G, TORIC>, dev, smem);
     if (e != cudaSuccess) return e;
-    scan_kernel<G><<<(unsigned)blocks, 32 * kScanWarps, smem, s>>>(p);
+    scan_kernel<G, TORIC><<<(unsigned)blocks, 32 * kScanWarps, smem, s>>>(p);
     return cudaGetLastError();
+}
+
+template <int G>
+cudaError_t launch_scan_g(const SweepParams& p, cudaStream_t s) {
+    return p.code ? launch_scan_t<G, true>(p, s) : launch_scan_t<G, false>(p, s);
 }
 
 }  // namespace
