@@ -311,6 +311,8 @@ int surfmcmc_autotune(surfmcmc_ctx* ctx, int32_t L, int32_t chains_per_class, do
  * annealing scaled to beta_j) and randomness key seed + j; <n> at beta = 0 is
  * 3/4 n_q (Sec. IV.A).  I_k = h/3 sum_j w_j <n>_{beta_j,k} (w = 1,4,2,..,4,1,
  * h = beta* / (n_beta-1)) in double precision, summed in order j = 0..n_beta-1.
+ * Grid points run side by side on streams of the context (forked from `stream`
+ * and joined to it) when one alone would not fill the device.
  *   n_beta        odd, 3..129 (21 in the paper).
  *   out_class     [n] int32 out: argmin_k I_k (= argmax Z_k), lowest on ties.
  *   out_log_z     [n][4] double out (may be NULL): log Z_k - max_k log Z_k

@@ -151,8 +151,8 @@ inline int widen_lanes_for(int sms, int L, int lam, long long n_bundles, int G, 
 
 // Thread budget of the one-block-per-bundle kernel (sweep_wide.cu) for a
 // launch; 0: the launch takes the throughput kernel.  Up to 4 bundles per
-// multiprocessor it is the faster one at every size measured (L = 5: 211
-// against 333 us for 60 sweeps, L = 25: 1618 against 1766); from 8 on it is
+// multiprocessor it is the faster one at every size measured (L = 5: 196
+// against 300 us for 60 sweeps, L = 25: 1212 against 1270); from 8 on it is
 // not.  The budget shares a multiprocessor's 1024 threads (64 registers
 // each) among its bundles.  at_once: launches of this shape that run at the
 // same time.

@@ -31,12 +31,11 @@
 // phase before; a thread adds its unoccupied words to a bit-sliced counter
 // after its stores, off the serial path.
 //
-// Measured (GB300, 4 x 4 chains, one bundle, us per phase, throughput kernel
-// with 32 lanes -> here): L = 5 1.07 -> 0.18, L = 13 2.25 -> 0.40, L = 25
-// 5.8 -> 1.2.  With 1, 2 and 4 bundles per multiprocessor a 60-sweep decode
-// takes 228, 305, 469 us against 653 at L = 13, and 681, 1014, 1618 against
-// 1756-1766 at L = 25; at 8 per multiprocessor the throughput kernel is as
-// fast or faster at every size, hence the limit in wide_batch (plan.cuh).
+// Measured (GB300, 4 x 4 chains): a 60-sweep decode with 1, 2 and 4 bundles per
+// multiprocessor takes 144, 231, 394 us at L = 13 against 524-531 on the
+// throughput kernel's best split, and 322, 638, 1212 against 1270 at L = 25; at
+// 8 per multiprocessor the throughput kernel is as fast or faster at every
+// size, hence the limit in wide_batch (plan.cuh).
 #include <algorithm>
 
 #include "sweep_kernel.cuh"
@@ -231,6 +230,12 @@ __device__ __forceinline__ uint32_t count_flush(uint32_t v[kWidePlanes], int lan
     return n;
 }
 
+// Word of qubit q in a plane: even qubits first, then odd ones.  Same-colour
+// generators of a row are two qubits apart, so their words lie on 32
+// different banks instead of 16 (one bundle per multiprocessor, 60 sweeps:
+// 228 -> 144 us at L = 13, 681 -> 322 at L = 25).
+__device__ __forceinline__ int word_of(int q, int nq) { return (q >> 1) + (q & 1 ? (nq + 1) >> 1 : 0); }
+
 template <int G, bool IND>
 __global__ void __launch_bounds__(kWideMaxThreads, 1) wide_kernel(const __grid_constant__ SweepParams p) {
     constexpr int SLOTS = PlaneBatch<G>::SLOTS, FIXED = wide_fixed<G>();
@@ -282,6 +287,9 @@ __global__ void __launch_bounds__(kWideMaxThreads, 1) wide_kernel(const __grid_c
             for (int k = 0; k < 4; ++k)
                 if (4 * (m - nc) + k < L) q[k] = untouched_qubit(L, col, 4 * (m - nc) + k);
         }
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (q[k] < nq) q[k] = word_of(q[k], nq);      // (the dummies stay behind the planes)
         tab[idx] = make_ushort4((unsigned short)q[0], (unsigned short)q[1], (unsigned short)q[2],
                                 (unsigned short)q[3]);
     }
@@ -290,8 +298,8 @@ __global__ void __launch_bounds__(kWideMaxThreads, 1) wide_kernel(const __grid_c
         for (int q = tid; q < nq; q += nt) {
             uint32_t xw, zw;
             start.word(q, xw, zw);
-            X[q] = xw;
-            Z[q] = zw;
+            X[word_of(q, nq)] = xw;
+            Z[word_of(q, nq)] = zw;
         }
     }
     // samples: the states after the phases of sweeps first .. t_end - 1
@@ -461,8 +469,8 @@ __global__ void __launch_bounds__(kWideMaxThreads, 1) wide_kernel(const __grid_c
     if (p.state_out) {
         uint32_t* st = p.state_out + gd.state_off + (size_t)bid * 2 * nq;
         for (int q = tid; q < nq; q += nt) {
-            st[q] = X[q];
-            st[nq + q] = Z[q];
+            st[q] = X[word_of(q, nq)];
+            st[nq + q] = Z[word_of(q, nq)];
         }
     }
     if (p.chain_frames) {
@@ -472,8 +480,8 @@ __global__ void __launch_bounds__(kWideMaxThreads, 1) wide_kernel(const __grid_c
             if (!((valid >> b) & 1u)) continue;
             uint32_t xw = 0, zw = 0;
             for (int k = 0; k < 32 && 32 * wi + k < nq; ++k) {
-                xw |= ((X[32 * wi + k] >> b) & 1u) << k;
-                zw |= ((Z[32 * wi + k] >> b) & 1u) << k;
+                xw |= ((X[word_of(32 * wi + k, nq)] >> b) & 1u) << k;
+                zw |= ((Z[word_of(32 * wi + k, nq)] >> b) & 1u) << k;
             }
             uint32_t* f = cfg + ci_of(b) * 2 * W;
             f[wi] = xw;
