@@ -295,7 +295,8 @@ void surfmcmc_plan_destroy(surfmcmc_plan* plan);
  * (the persistent grid; a cap above what fits counts as no cap), and records
  * the fastest pair in ctx for later calls with lanes_per_bundle = 0 and the
  * same (L, chains_per_class); ragged calls use the entry of their heaviest
- * size.  Results never depend on the choice.  *best_lanes and
+ * size.  (Batches of up to 4 bundles per multiprocessor run one block per
+ * bundle whatever was tuned.)  Results never depend on the choice.  *best_lanes and
  * *best_blocks_per_sm receive it, ms[SURFMCMC_TUNE_LANES][SURFMCMC_TUNE_BLOCKS]
  * the timings in milliseconds (NaN where the shape does not fit); any of the
  * three may be NULL.  EINVAL for bad arguments. */
