@@ -1133,10 +1133,9 @@ int surfmcmc_ragged_plan_create(surfmcmc_ctx* ctx, const int32_t* Ls, const uint
     cudaStream_t cap;
     if ((e = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking)) != cudaSuccess)
         return cleanup(fail(ctx, SURFMCMC_ECUDA, "stream: %s", cudaGetErrorString(e)));
-    if ((rc = ragged_upload(ctx, lay, n, rs, cap)) ||
-        (e = prepare_sweep(lay.sp, lay.lam)) != cudaSuccess) {
+    if ((rc = ragged_upload(ctx, lay, n, rs, cap))) {
         cudaStreamDestroy(cap);
-        return cleanup(rc ? rc : fail(ctx, SURFMCMC_ECUDA, "prepare: %s", cudaGetErrorString(e)));
+        return cleanup(rc);
     }
     const bool timing = ctx->timing;
     ctx->timing = false;  // no event nodes in the graph

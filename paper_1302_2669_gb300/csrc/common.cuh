@@ -294,8 +294,6 @@ cudaError_t launch_sweep_modes_flips(const SweepParams& p, int lanes_per_bundle,
 cudaError_t launch_sweep_scan(const SweepParams& p, cudaStream_t s);
 // The launch with one block per bundle (colour sweeps without accept counts).
 cudaError_t launch_sweep_wide(const SweepParams& p, cudaStream_t s);
-cudaError_t prepare_sweep_flips(const SweepParams& p, int lanes_per_bundle);
-cudaError_t prepare_sweep(const SweepParams& p, int lanes_per_bundle);
 size_t sweep_smem_bytes(int nq, int nc, int lanes_per_bundle);  // dynamic shared memory of a block
 long long sweep_units(long long n_bundles, int lanes_per_bundle);  // work units of a group
 cudaError_t launch_gen_syndromes(uint64_t seed, uint32_t id0, long long n, int L, double p,

@@ -14,12 +14,6 @@ size_t sweep_smem_bytes(int nq, int nc, int lam) {
 long long sweep_units(long long n_bundles, int lam) { return (n_bundles + (long long)kWarps * (32 / lam) - 1) /
                                                                ((long long)kWarps * (32 / lam)); }
 
-// Sets the kernel's shared-memory limit ahead of a stream capture.
-cudaError_t prepare_sweep(const SweepParams& p, int lam) {
-    if (p.scan || p.wide) return cudaSuccess;   // their launchers raise it themselves
-    return p.noise == 1 ? prepare_sweep_flips(p, lam) : prepare_noise<false>(p, lam);
-}
-
 cudaError_t launch_sweep(const SweepParams& p, int lam, cudaStream_t s) {
     if (p.scan) return launch_sweep_scan(p, s);
     if (p.wide) return launch_sweep_wide(p, s);

@@ -4,8 +4,6 @@
 
 namespace surfmcmc {
 
-cudaError_t prepare_sweep_flips(const SweepParams& p, int lam) { return prepare_noise<true>(p, lam); }
-
 cudaError_t launch_sweep_flips(const SweepParams& p, int lam, cudaStream_t s) {
     return launch_noise<true>(p, lam, s);
 }

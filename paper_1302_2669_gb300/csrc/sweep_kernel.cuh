@@ -903,9 +903,11 @@ __global__ void __launch_bounds__(128, sweep_blocks_per_sm(G, LAM)) sweep_kernel
 constexpr int kWarps = 4;
 
 // The dynamic shared-memory limit of one kernel instantiation, raised on
-// demand.  The attribute belongs to the current device's context, so the
+// demand (also inside a stream capture, where setting a function attribute is
+// allowed).  The attribute belongs to the current device's context, so the
 // limit already set is kept per device, under a lock (contexts on several
-// host threads may launch at once).
+// host threads may launch at once).  Nothing else sets the attribute: a
+// smaller value written past this record would fail the next large launch.
 struct SmemLimit {
     static constexpr int kMaxDevices = 64;
     std::mutex m;
@@ -950,36 +952,6 @@ static cudaError_t launch_t(const SweepParams& p, cudaStream_t s) {
     }
     sweep_kernel<G, LAM, IND, ACPT, HM><<<(unsigned)blocks, 32 * kWarps, smem, s>>>(p);
     return cudaGetLastError();
-}
-
-template <int G, int LAM, bool IND>
-static cudaError_t prepare_t(const SweepParams& p) {
-    const size_t smem = sweep_smem_bytes(p.grp_nq_max, p.grp_nc_max, LAM);
-    return cudaFuncSetAttribute(sweep_kernel<G, LAM, IND, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)smem);
-}
-
-template <int G, bool IND>
-static cudaError_t prepare_g(const SweepParams& p, int lam) {
-    switch (lam) {
-        case 2: return prepare_t<G, 2, IND>(p);
-        case 4: return prepare_t<G, 4, IND>(p);
-        case 8: return prepare_t<G, 8, IND>(p);
-        case 16: return prepare_t<G, 16, IND>(p);
-        case 32: return prepare_t<G, 32, IND>(p);
-        default: return cudaErrorInvalidValue;
-    }
-}
-
-template <bool IND>
-static cudaError_t prepare_noise(const SweepParams& p, int lam) {
-    switch (p.G) {
-        case 4: return prepare_g<4, IND>(p, lam);
-        case 8: return prepare_g<8, IND>(p, lam);
-        case 16: return prepare_g<16, IND>(p, lam);
-        case 32: return prepare_g<32, IND>(p, lam);
-        default: return cudaErrorInvalidValue;
-    }
 }
 
 template <int G, bool IND>
