@@ -381,7 +381,10 @@ void surfmcmc_server_destroy(surfmcmc_server* server);
  * sweep kernel.  surfmcmc_sweep_time waits for the recorded events, returns
  * in *ms the summed sweep-kernel time in milliseconds and in *launches the
  * number of sweep launches since the previous query (either pointer may be
- * NULL), and clears the record.  EINVAL for a NULL ctx. */
+ * NULL), and clears the record.  Where surfmcmc_decode_ti runs grid points
+ * side by side their launches overlap, so one pair on its stream spans them
+ * all (with the grid points' small means kernels between them): their time
+ * counts once, their launches each.  EINVAL for a NULL ctx. */
 int surfmcmc_set_timing(surfmcmc_ctx* ctx, int enable);
 int surfmcmc_sweep_time(surfmcmc_ctx* ctx, double* ms, int64_t* launches);
 

@@ -23,6 +23,13 @@ struct Tuned {
     int blocks_per_sm = 0;   // persistent blocks per multiprocessor (0: as many as fit)
 };
 
+// Events around sweep launches (surfmcmc_set_timing): one launch, or several
+// that run at the same time.
+struct TimedSpan {
+    cudaEvent_t first = nullptr, second = nullptr;
+    int64_t launches = 1;
+};
+
 struct surfmcmc_ctx {
     int device = 0;
     int sms = 0;               // multiprocessors of the device
@@ -31,8 +38,8 @@ struct surfmcmc_ctx {
     std::string last_error;
     bool timing = false;
     std::map<std::pair<int, int>, Tuned> tuned;  // (L, chains per class) -> launch shape
-    std::vector<std::pair<cudaEvent_t, cudaEvent_t>> pending;  // recorded around sweep launches
-    std::vector<std::pair<cudaEvent_t, cudaEvent_t>> spare;
+    std::vector<TimedSpan> pending;  // recorded around sweep launches
+    std::vector<TimedSpan> spare;
     // side streams of decode_ti's grid points and their events (start, done);
     // created on first use
     std::vector<cudaStream_t> side;
@@ -293,7 +300,7 @@ struct SweepIO {
     unsigned int* unit_counter = nullptr;  // work queue of the persistent kernel
 };
 
-int record_start(surfmcmc_ctx* ctx, std::pair<cudaEvent_t, cudaEvent_t>* ev, cudaStream_t s) {
+int record_start(surfmcmc_ctx* ctx, TimedSpan* ev, cudaStream_t s) {
     if (!ctx->timing) return SURFMCMC_OK;
     if (!ctx->spare.empty()) {
         *ev = ctx->spare.back();
@@ -306,9 +313,10 @@ int record_start(surfmcmc_ctx* ctx, std::pair<cudaEvent_t, cudaEvent_t>* ev, cud
     return SURFMCMC_OK;
 }
 
-int record_end(surfmcmc_ctx* ctx, std::pair<cudaEvent_t, cudaEvent_t> ev, cudaStream_t s) {
+int record_end(surfmcmc_ctx* ctx, TimedSpan ev, cudaStream_t s, int64_t launches = 1) {
     if (!ctx->timing) return SURFMCMC_OK;
     CK(cudaEventRecord(ev.second, s));
+    ev.launches = launches;
     ctx->pending.push_back(ev);
     return SURFMCMC_OK;
 }
@@ -338,7 +346,7 @@ int run_segments(surfmcmc_ctx* ctx, SweepParams sp, const std::vector<std::vecto
         sp.chain_n = last ? io.chain_n : nullptr;
         sp.chain_frames = last ? io.chain_frames : nullptr;
         sp.unit_counter = io.unit_counter;
-        std::pair<cudaEvent_t, cudaEvent_t> ev{nullptr, nullptr};
+        TimedSpan ev;
         if ((rc = record_start(ctx, &ev, s))) return rc;
         CK(launch_sweep(sp, lam, s));
         if ((rc = record_end(ctx, ev, s))) return rc;
@@ -674,7 +682,7 @@ int surfmcmc_sweep_time(surfmcmc_ctx* ctx, double* ms, int64_t* launches) {
         CK(cudaEventSynchronize(e.second));
         CK(cudaEventElapsedTime(&t, e.first, e.second));
         total += t;
-        ++count;
+        count += e.launches;
         ctx->spare.push_back(e);
     }
     ctx->pending.clear();
@@ -1006,9 +1014,13 @@ int surfmcmc_decode_ti(surfmcmc_ctx* ctx, const uint8_t* syndromes, int64_t n, i
             if ((rc = grid_point(j, 0, s))) return rc;
     } else {
         // fork from the caller's stream and join it again, also after an error
-        // (the side streams work on the context's scratch)
+        // (the side streams work on the context's scratch).  The launches of
+        // different streams overlap, so their time is one span from fork to join.
+        TimedSpan ev;
+        if ((rc = record_start(ctx, &ev, s))) return rc;
         CK(cudaEventRecord(ctx->side_start, s));
-        rc = SURFMCMC_OK;
+        const bool timing = ctx->timing;
+        ctx->timing = false;
         int forked = 0;
         for (; forked < S && !rc; ++forked)
             if (cudaStreamWaitEvent(ctx->side[forked], ctx->side_start, 0) != cudaSuccess)
@@ -1018,7 +1030,8 @@ int surfmcmc_decode_ti(surfmcmc_ctx* ctx, const uint8_t* syndromes, int64_t n, i
             if ((cudaEventRecord(ctx->side_done[i], ctx->side[i]) != cudaSuccess ||
                  cudaStreamWaitEvent(s, ctx->side_done[i], 0) != cudaSuccess) && !rc)
                 rc = fail(ctx, SURFMCMC_ECUDA, "side stream: %s", cudaGetErrorString(cudaGetLastError()));
-        if (rc) return rc;
+        ctx->timing = timing;
+        if (rc || (rc = record_end(ctx, ev, s, (int64_t)(N - 1) * (int64_t)segs0.size()))) return rc;
     }
     uint64_t T[33];
     double beta_bar;
