@@ -183,14 +183,19 @@ __host__ __device__ __forceinline__ int geo_nc(int code, int L) { return code ? 
 __host__ __device__ __forceinline__ int padded_nq(int nq, int lam) { return (nq + 4 * lam - 1) / (4 * lam) * (4 * lam); }
 __host__ __device__ __forceinline__ int bundle_stride(int nq, int lam) { return 2 * (padded_nq(nq, lam) + 2) + 1; }
 
-// Blocks per SM the sweep kernel is compiled for (its register bound): 6
-// (80 registers) with planes of 32 and 16 chains, 3 with narrower planes.  On
-// 32-chain planes 5 blocks took 10.45 ms where 6 take 10.04 (36,480 syndromes
-// at L = 13, 40 sweeps).  On 16-chain planes the kernels of 32 and 8 lanes
-// spill at 80 registers and are faster at 5 (L = 25: 5.55 against 5.68 ms, L =
-// 9: 6.30 against 6.62); those of 16 lanes are not (L = 13: 5.74 against 5.49).
+// Blocks per SM the sweep kernel is compiled for (its register bound): 5 (96
+// registers) with planes of 32 chains, 5 or 6 (80) with 16, 3 with narrower
+// planes.  At 80 registers the 32-chain kernels spill up to 92 bytes: over L =
+// 3 .. 31 and 638 to 36,480 bundles 6 blocks are 8, 10, 5, 5 and 1.5 % slower
+// than 5 on average at 2, 4, 8, 16 and 32 lanes, also where shared memory lets
+// no sixth block in (16,384 syndromes of 64 chains at L = 17: 12.41 against
+// 11.91 ms for 60 sweeps); near whole waves of 6 they are ahead by a little
+// (36,480 syndromes at L = 13: 14.55 against 14.71).  On 16-chain planes the
+// kernels of 32 and 8 lanes spill at 80 registers and are faster at 5 (L = 25:
+// 5.55 against 5.68 ms, L = 9: 6.30 against 6.62); those of 16 lanes are not
+// (L = 13: 5.74 against 5.49).
 __host__ __device__ constexpr int sweep_blocks_per_sm(int G, int lam) {
-    return G == 16 && (lam == 32 || lam == 8) ? 5 : G >= 16 ? 6 : 3;
+    return G == 32 || (G == 16 && (lam == 32 || lam == 8)) ? 5 : G == 16 ? 6 : 3;
 }
 
 // ---------------------------------------------------------------------------
