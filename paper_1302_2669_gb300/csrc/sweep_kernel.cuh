@@ -549,8 +549,7 @@ struct BundleMap {
 };
 
 // Index of the chain behind valid bit b of bundle `bid` in the [items][C]
-// arrays; from the bundle's number alone, for the places where keeping its
-// map would hold registers through the sweeps.
+// arrays; from the bundle's number alone, where its map is not kept (keep_map).
 template <int G>
 __device__ __forceinline__ size_t chain_index(const SweepParams& p, const GroupDesc& gd, long long bid, int b) {
     if constexpr (G == 32) {
@@ -634,6 +633,19 @@ struct StartState {
     }
 };
 
+// Whether the sweeps keep the bundle's map (its syndromes and ids) in
+// registers, or read it back from shared memory and work the chains' indices
+// out anew.  Averages over L = 3 .. 31 and 638 to 36,480 bundles: keeping it
+// is 1.5 to 6 % faster with 8-chain planes (four ids, no register shortage),
+// 1 % with 32-chain planes (one id; 4 % slower at 4 lanes) and 5 % with
+// 16-chain planes at 4 lanes; with 16-chain planes otherwise it costs 1 to 8
+// %, with 4-chain planes (eight ids) up to 2 %.  Counting accepts on 32-chain
+// planes takes 15 % longer without it (L = 25, 912 syndromes of 32 chains, 60
+// sweeps: 5.21 ms against 3.91).
+__host__ __device__ constexpr bool keep_map(int G, int lam) {
+    return G == 8 || (G == 32 && lam != 4) || (G == 16 && lam == 4);
+}
+
 template <int G, int LAM, bool IND, bool ACPT, int HM>
 __device__ __forceinline__ void run_unit(const SweepParams& p, const GroupDesc& gd, long long unit,
                                          uint32_t* smem, const ushort4* tab) {
@@ -659,14 +671,10 @@ __device__ __forceinline__ void run_unit(const SweepParams& p, const GroupDesc& 
     uint32_t* fx = fixed + (warp * B + slot) * kHeadFixedWords;
     const int W = gd.W;
     uint32_t* cfg = p.chain_frames ? p.chain_frames + gd.frames_off - (size_t)gd.item_base * p.C * 2 * W : nullptr;
-    uint32_t valid;
+    const BundleMap<G> bm(p, gd, bid);
+    const uint32_t valid = bm.valid;
+    constexpr bool KEEP = keep_map(G, LAM);
     {
-        // The bundle's map lives for the prologue only: kept through the
-        // sweeps its syndromes and ids hold registers that these need (10.04
-        // ms against 10.34 without, 36,480 syndromes at L = 13, 64 chains, 40
-        // sweeps; 7.43 against 7.60 at L = 17, 16 chains).
-        const BundleMap<G> bm(p, gd, bid);
-        valid = bm.valid;
         if (sub == 0) {
             binfo[slot * (kMaxSlots + 1)] = bm.w;
 #pragma unroll
@@ -686,7 +694,9 @@ __device__ __forceinline__ void run_unit(const SweepParams& p, const GroupDesc& 
         X[nqp + 1] = 0xFFFFFFFFu; Z[nqp + 1] = 0u;  // dummy of sigma_z generators
     }
     // Owned chains' sums live in the output array; flushes add to them.
-    auto ci_of = [&](int b) -> size_t { return chain_index<G>(p, gd, bid, b); };
+    auto ci_of = [&](int b) -> size_t {
+        return KEEP ? (size_t)bm.syn_of(b) * p.C + bm.chain_of(b) : chain_index<G>(p, gd, bid, b);
+    };
 #pragma unroll
     for (int j = 0; j < NJ; ++j) {
         const int b = sub + j * LAM;
@@ -715,6 +725,7 @@ __device__ __forceinline__ void run_unit(const SweepParams& p, const GroupDesc& 
             if (lane == 0) *q_cnt = 0u;
             __syncwarp();
             const uint32_t* info = binfo + slot * (kMaxSlots + 1);   // w, ids
+            const uint32_t* ids = KEEP ? bm.sid : info + 1;
             if (active) {
                 for (int m = sub; m < nc; m += LAM) {
                     const ushort4 sp = tc[m];
@@ -748,7 +759,7 @@ __device__ __forceinline__ void run_unit(const SweepParams& p, const GroupDesc& 
                             // Delta n - 1 = E0 + 2 E1 on the uphill chains
                             const uint32_t E0 = ~w0, E1 = Z0 & Wge3;
                             const uint32_t cm = colm | (uint32_t)m;
-                            acc |= bernoulli_range<G, 0, HEAD, HM>(p, U, E0, E1, info + 1, info[0], t, cm, fx);
+                            acc |= bernoulli_range<G, 0, HEAD, HM>(p, U, E0, E1, ids, KEEP ? bm.w : info[0], t, cm, fx);
                             if constexpr (HEAD < NBATCH) {
                                 if (U) {
                                     const uint32_t qi = atomicAdd(q_cnt, 1u);
@@ -761,7 +772,8 @@ __device__ __forceinline__ void run_unit(const SweepParams& p, const GroupDesc& 
                                         it[4] = acc;
                                         continue;  // flipped after the queue is resolved
                                     }
-                                    acc |= bernoulli_range<G, HEAD, NBATCH, HM>(p, U, E0, E1, info + 1, info[0], t, cm);
+                                    acc |= bernoulli_range<G, HEAD, NBATCH, HM>(p, U, E0, E1, ids, KEEP ? bm.w : info[0], t,
+                                                                                cm);
                                 }
                             }
                         }
