@@ -105,17 +105,19 @@ constexpr size_t kSweepSmemLimit = 200 * 1024;
 
 // Lanes per bundle by rule, for `bundles` bundles on a device with `sms`
 // multiprocessors: the smallest modelled time of a colour phase.  A unit
-// (4 warps x 32/lam bundles) takes rounds + 1.6 per phase: its proposals'
+// (4 warps x 32/lam bundles) takes rounds + 1.35 per phase: its proposals'
 // rounds and what every phase costs besides (queue pass, counting).  One
 // block alone on a multiprocessor runs at its latency, each further one adds
-// a third of that; the units past full waves of the r blocks that fit overlap
+// 1/2.75 of that; the units past full waves of the r blocks that fit overlap
 // with them by half when they are few, not at all when they are nearly a
 // wave.  Fewer lanes fill the rounds and the queue better (at a cost in bank
-// conflicts and frames: 4, 20 and 24 % at 8, 4 and 2 lanes), more lanes make
-// short units for batches that do not fill the device.  Fitted to every split
-// of L = 3 .. 25 at 2,048 to 73,000 bundles: the pick is within 6 % of the
-// fastest.  (The fill of the last round alone lost up to 97 %: 2 lanes for
-// 8,192 bundles at L = 5 and 7.)  The results do not depend on the lanes.
+// conflicts, frames and longer units: 6 % at 16 lanes, 15 % below), more lanes
+// make short units for batches that do not fill the device.  Fitted to every
+// split of L = 3 .. 31 (torus 4 .. 30), all plane widths and both noise models,
+// at 638 to 36,480 bundles: the pick is 0.5 % off the fastest split on average
+// and within 8.5 % of it in 99 of 100 of those 1,558 shapes (at most 20 % off
+// on 4-chain planes, 12 % on the others).  The results do not depend on the
+// lanes.
 inline int choose_lanes(int sms, int L, long long bundles, int G, int code) {
     const int nq = geo_nq(code, L), nc = geo_nc(code, L);
     int best = 32;
@@ -127,9 +129,9 @@ inline int choose_lanes(int sms, int L, long long bundles, int G, int code) {
         const double r = fit < 1 ? 1 : fit < sweep_blocks_per_sm(G, lam) ? fit : sweep_blocks_per_sm(G, lam);
         const double u = (double)sweep_units(bundles, lam) / (sms > 0 ? sms : 1);
         const double full = std::floor(u / r), rest = u - full * r;
-        const double tail = rest > 0 ? (3.0 + rest) * (0.5 + 0.5 * rest / r) : 0.0;
-        const double waves = full > 0 ? full * (3.0 + r) + tail : 3.0 + std::ceil(u);
-        const double cost = (rounds + 1.6) * waves * (lam == 2 ? 1.24 : lam == 4 ? 1.20 : lam == 8 ? 1.04 : 1.0);
+        const double tail = rest > 0 ? (2.75 + rest) * (0.5 + 0.5 * rest / r) : 0.0;
+        const double waves = full > 0 ? full * (2.75 + r) + tail : 2.75 + std::ceil(u);
+        const double cost = (rounds + 1.35) * waves * (lam < 16 ? 1.15 : lam == 16 ? 1.06 : 1.0);
         if (cost < best_cost) {
             best_cost = cost;
             best = lam;
