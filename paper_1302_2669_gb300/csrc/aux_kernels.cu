@@ -176,22 +176,28 @@ cudaError_t launch_gen_syndromes_toric(uint64_t seed, uint32_t id0, long long n,
 
 // Pure error: a straight string from every anyon to its nearer absorbing
 // boundary (Sec. III), s-anyons vertically (z string), p-anyons horizontally
-// (x string); ties go up/left.  One warp per syndrome: the strings touch the
-// qubits of the even grid rows only, lane i holding row 2i of both planes as
-// an L-bit word (bit j: column 2j).  The syndrome's rows become such words by
-// ballots; a z string up (down) from row a covers the rows i <= a (i > a), so
-// the z plane is the suffix (prefix) xor of the row words over the lanes, and
-// the x plane the same over the bits of a word.  (One thread per syndrome
-// walking its strings took 35 us for one syndrome at L = 13 and 300 us at
-// L = 25, all latency.)
+// (x string); ties go up/left.  WD >= L lanes of a warp per syndrome (a null
+// one: s is not read): the strings touch the qubits of the even grid rows only,
+// lane i holding row 2i of both planes as an L-bit word (bit j: column 2j).
+// The syndrome's rows become such words by ballots; a z string up (down) from
+// row a covers the rows i <= a (i > a), so the z plane is the suffix (prefix)
+// xor of the row words over the lanes, and the x plane the same over the bits
+// of a word.  (One thread per syndrome walking its strings took 35 us for one
+// syndrome at L = 13 and 300 us at L = 25, all latency.)
+template <int WD>
 __device__ __forceinline__ void pure_error_rows(int L, const uint8_t* s, int lane, uint32_t& xrow, uint32_t& zrow) {
     const uint32_t full = 0xffffffffu;
+    const int first = (threadIdx.x & 31) & ~(WD - 1);   // the syndrome's lane 0
     uint32_t sx = 0, sz = 0;   // lane a: row a of the sigma_x and of the sigma_z generators
 #pragma unroll 4
     for (int a = 0; a < L; ++a) {
-        const bool dx = a < L - 1 && lane < L && s[a * L + lane] != 0;
-        const bool dz = lane < L - 1 && s[L * (L - 1) + a * (L - 1) + lane] != 0;
-        const uint32_t wx = __ballot_sync(full, dx), wz = __ballot_sync(full, dz);
+        const bool dx = s && a < L - 1 && lane < L && s[a * L + lane] != 0;
+        const bool dz = s && lane < L - 1 && s[L * (L - 1) + a * (L - 1) + lane] != 0;
+        uint32_t wx = __ballot_sync(full, dx), wz = __ballot_sync(full, dz);
+        if constexpr (WD < 32) {
+            wx = (wx >> first) & ((1u << WD) - 1u);
+            wz = (wz >> first) & ((1u << WD) - 1u);
+        }
         if (lane == a) {
             sx = wx;
             sz = wz;
@@ -200,18 +206,18 @@ __device__ __forceinline__ void pure_error_rows(int L, const uint8_t* s, int lan
     // s-anyons of row a go up if 2 (a + 1) <= L
     uint32_t up = 2 * (lane + 1) <= L ? sx : 0u, down = 2 * (lane + 1) <= L ? 0u : sx;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t u = __shfl_down_sync(full, up, o), d = __shfl_up_sync(full, down, o);
-        if (lane + o < 32) up ^= u;
+    for (int o = 1; o < WD; o <<= 1) {
+        const uint32_t u = __shfl_down_sync(full, up, o, WD), d = __shfl_up_sync(full, down, o, WD);
+        if (lane + o < WD) up ^= u;
         if (lane >= o) down ^= d;
     }
-    down = __shfl_up_sync(full, down, 1);       // rows below the anyon's
+    down = __shfl_up_sync(full, down, 1, WD);   // rows below the anyon's
     zrow = up ^ (lane > 0 ? down : 0u);
     // p-anyons of column b go left if 2 (b + 1) <= L: bits j <= b; else j > b
     const uint32_t lmask = (1u << (L / 2)) - 1u;
     uint32_t left = sz & lmask, right = sz & ~lmask;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
+    for (int o = 1; o < WD; o <<= 1) {
         left ^= left >> o;
         right ^= right << o;
     }
@@ -220,11 +226,13 @@ __device__ __forceinline__ void pure_error_rows(int L, const uint8_t* s, int lan
     if (lane >= L) xrow = 0u;
 }
 
-// Writes the frame of the row words (f: [2][W]) and returns its class code
-// a + 2b (x parity on column 0, z parity on row 0).  sh: 2 kMaxWords words.
+// Writes the frame of the row words (f: [2][W], or NULL: nothing) and returns
+// its class code a + 2b (x parity on column 0, z parity on row 0).  sh: 2 W
+// words.
+template <int WD>
 __device__ __forceinline__ int write_rows(int L, int W, uint32_t xrow, uint32_t zrow, int lane, uint32_t* sh,
                                           uint32_t* f) {
-    for (int w = lane; w < 2 * W; w += 32) sh[w] = 0u;
+    for (int w = lane; w < 2 * W; w += WD) sh[w] = 0u;
     __syncwarp();
     if (lane < L) {
         const int q = lane * (2 * L - 1), w = q >> 5, o = q & 31;
@@ -235,24 +243,30 @@ __device__ __forceinline__ int write_rows(int L, int W, uint32_t xrow, uint32_t 
         if (z >> 32) atomicOr(&sh[W + w + 1], (uint32_t)(z >> 32));
     }
     __syncwarp();
-    for (int w = lane; w < 2 * W; w += 32) f[w] = sh[w];
-    const int a = __popc(__ballot_sync(0xffffffffu, xrow & 1u)) & 1;
-    const int b = __popc(__shfl_sync(0xffffffffu, zrow, 0)) & 1;
-    return a + 2 * b;
+    for (int w = lane; f && w < 2 * W; w += WD) f[w] = sh[w];
+    uint32_t column = __ballot_sync(0xffffffffu, xrow & 1u);
+    if constexpr (WD < 32) column = (column >> ((threadIdx.x & 31) & ~(WD - 1))) & ((1u << WD) - 1u);
+    const int b = __popc(__shfl_sync(0xffffffffu, zrow, 0, WD)) & 1;
+    return (__popc(column) & 1) + 2 * b;
 }
 
 constexpr int kStartWarps = 4;
 
+// 32 / WD syndromes per warp: small codes would leave most of a warp's lanes
+// idle (65,536 syndromes at L = 5: 51 us with a whole warp each, 35 with 8
+// lanes; one thread each took 35; one syndrome takes the same time at any WD).
+template <int WD>
 __global__ void __launch_bounds__(32 * kStartWarps) start_frames_kernel(const uint8_t* syn, long long n, int L,
                                                                         uint32_t* frames, int32_t* code) {
-    __shared__ uint32_t sh[kStartWarps][2 * kMaxWords];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, W = n_words(L);
-    const long long i = (long long)blockIdx.x * kStartWarps + warp;
-    if (i >= n) return;
+    constexpr int S = 32 / WD;
+    __shared__ uint32_t sh[kStartWarps * S][2 * ((2 * WD * WD - 2 * WD + 1 + 31) / 32)];   // planes of L <= WD
+    const int sub = threadIdx.x / WD, lane = threadIdx.x % WD, W = n_words(L);
+    const long long i = (long long)blockIdx.x * kStartWarps * S + sub;
+    const bool mine = i < n;   // the warp's last syndromes may be missing
     uint32_t x, z;
-    pure_error_rows(L, syn + i * n_stabs(L), lane, x, z);
-    const int c = write_rows(L, W, x, z, lane, sh[warp], frames + i * 2 * W);
-    if (code && lane == 0) code[i] = c;
+    pure_error_rows<WD>(L, mine ? syn + i * n_stabs(L) : nullptr, lane, x, z);
+    const int c = write_rows<WD>(L, W, x, z, lane, sh[sub], mine ? frames + i * 2 * W : nullptr);
+    if (mine && code && lane == 0) code[i] = c;
 }
 
 // Ragged batches: pure errors, class codes and ids of every item in one
@@ -268,8 +282,8 @@ __global__ void __launch_bounds__(32 * kStartWarps) start_ragged_kernel(const __
     const int L = p.L[g], W = n_words(L);
     const long long o = p.perm[i];
     uint32_t x, z;
-    pure_error_rows(L, p.src + p.src_off[o], lane, x, z);
-    const int c = write_rows(L, W, x, z, lane, sh[warp], p.e0 + p.e0_off[g] + (i - p.item_base[g]) * 2 * W);
+    pure_error_rows<32>(L, p.src + p.src_off[o], lane, x, z);
+    const int c = write_rows<32>(L, W, x, z, lane, sh[warp], p.e0 + p.e0_off[g] + (i - p.item_base[g]) * 2 * W);
     if (lane == 0) {
         p.code[i] = c;
         p.ids_out[i] = p.ids ? p.ids[o] : p.id0 + (uint32_t)o;
@@ -585,15 +599,26 @@ cudaError_t launch_gen_syndromes(uint64_t seed, uint32_t id0, long long n, int L
     return cudaGetLastError();
 }
 
+template <int WD>
+static void start_frames_planar(const uint8_t* syn, long long n, int L, uint32_t* frames, int32_t* code,
+                                cudaStream_t s) {
+    constexpr int per_block = kStartWarps * (32 / WD);
+    start_frames_kernel<WD><<<(unsigned)((n + per_block - 1) / per_block), 32 * kStartWarps, 0, s>>>(syn, n, L, frames,
+                                                                                                     code);
+}
+
 cudaError_t launch_start_frames(const uint8_t* syn, long long n, int L, uint32_t* frames, int32_t* code,
                                 cudaStream_t s, int toric) {
     if (n == 0) return cudaSuccess;
     const int bs = 128;
     if (toric)
         start_frames_toric_kernel<<<(unsigned)((n + bs - 1) / bs), bs, 0, s>>>(syn, n, L, frames, code);
+    else if (L <= 8)
+        start_frames_planar<8>(syn, n, L, frames, code, s);
+    else if (L <= 16)
+        start_frames_planar<16>(syn, n, L, frames, code, s);
     else
-        start_frames_kernel<<<(unsigned)((n + kStartWarps - 1) / kStartWarps), 32 * kStartWarps, 0, s>>>(syn, n, L,
-                                                                                                         frames, code);
+        start_frames_planar<32>(syn, n, L, frames, code, s);
     return cudaGetLastError();
 }
 
