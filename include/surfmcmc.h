@@ -369,7 +369,8 @@ int surfmcmc_server_poll(surfmcmc_server* server, int64_t max_results, uint32_t*
 /* Counters since creation: requests admitted to batches, batches launched,
  * times admission had to wait for memory (a free slot and waiting requests,
  * but not even one request's scratch fits the budget next to the batches in
- * flight; counted once per wait), requests waiting now. */
+ * flight; counted once per wait, also while the waiting requests are fewer
+ * than max_batch and younger than max_wait_us), requests waiting now. */
 int surfmcmc_server_stats(surfmcmc_server* server, int64_t* admitted, int64_t* batches, int64_t* memory_stalls,
                           int64_t* pending);
 
