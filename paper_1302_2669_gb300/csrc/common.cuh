@@ -293,6 +293,7 @@ cudaError_t launch_sweep_flips(const SweepParams& p, int lanes_per_bundle, cudaS
 // The launch on a kernel with its digit-plane modes compiled in;
 // cudaErrorNotSupported (nothing launched) where there is none.
 cudaError_t launch_sweep_modes(const SweepParams& p, int lanes_per_bundle, cudaStream_t s);
+cudaError_t launch_sweep_modes_16(const SweepParams& p, int lanes_per_bundle, cudaStream_t s);
 cudaError_t launch_sweep_modes_narrow(const SweepParams& p, int lanes_per_bundle, cudaStream_t s);
 cudaError_t launch_sweep_modes_flips(const SweepParams& p, int lanes_per_bundle, cudaStream_t s);
 // Random scan (sweep_scan.cu).

@@ -347,23 +347,25 @@ __device__ __forceinline__ void head_fixed_words(const SweepParams& p, const uin
 // Digit-plane modes of a launch, per quad of planes: 0 every threshold digit
 // is 0, 1 only T[1] has nonzero digits, 3 only T[1] and T[2], 2 general (right
 // for any digits).  The quads after the first two run as general; the first
-// two run in one of three patterns, (0, 1), (1, 3) and (2, 2), each with
-// kernels of its own (HM = 1, 2, 3), chosen as the first that covers the
-// launch's modes: the sampled sweeps at p = 0.08-0.15 take (0, 1), those up
-// to 0.18 (1, 3; 3.5 % faster than as (1, 2)), hot annealing stages (2, 2).  HM = 0 reads the modes from
-// the launch parameters (accept-all and reject-all launches, accept counts,
-// the shapes without kernels of their own).
+// two run in one of four patterns, each with kernels of its own, chosen as the
+// first that covers the launch's modes: (0, 1) (HM = 1) at p = 0.08-0.15, (1, 3)
+// (HM = 2) up to 0.18, 3.5 % faster than as (1, 2), and in annealing stages
+// (1, 2) (HM = 4; the annealed burn-in of 16,384 syndromes at L = 13, 64 chains,
+// 200 sweeps: 24.0 ms, and 24.5 with those stages as (2, 2)) and in the hottest
+// ones (2, 2) (HM = 3).  HM = 0 reads the modes from the launch parameters
+// (accept-all and reject-all launches, accept counts, the shapes without
+// kernels of their own).
 template <int HM>
 __device__ __forceinline__ uint32_t quad_mode(const SweepParams& p, int q) {
     if constexpr (HM == 0) return (p.qmodes >> (2 * q)) & 3u;
-    else return q >= 2 || HM == 3 ? 2u : HM == 1 ? (q == 0 ? 0u : 1u) : (q == 0 ? 1u : 3u);
+    else return q >= 2 || HM == 3 ? 2u : HM == 1 ? (q == 0 ? 0u : 1u) : q == 0 ? 1u : HM == 2 ? 3u : 2u;
 }
 
 // The specialised head pattern of a launch (0: none).
 __host__ __device__ inline int head_pattern(const SweepParams& p) {
     if (p.accept_all || p.reject_all) return 0;
     const uint32_t m0 = p.qmodes & 3u, m1 = (p.qmodes >> 2) & 3u;
-    return m0 == 0 && m1 <= 1 ? 1 : m0 <= 1 && m1 != 2 ? 2 : 3;
+    return m0 == 0 && m1 <= 1 ? 1 : m0 <= 1 ? (m1 != 2 ? 2 : 4) : 3;
 }
 
 // Accept mask of the undecided uphill chains U (all have Delta n = d > 0,

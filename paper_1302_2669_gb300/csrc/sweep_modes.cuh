@@ -26,15 +26,19 @@ static cudaError_t launch_g_hm(const SweepParams& p, int lam, cudaStream_t s) {
         case 1: return launch_hm<G, IND, 1>(p, lam, s);
         case 2: return launch_hm<G, IND, 2>(p, lam, s);
         case 3: return launch_hm<G, IND, 3>(p, lam, s);
+        case 4: return launch_hm<G, IND, 4>(p, lam, s);
         default: return cudaErrorNotSupported;
     }
 }
 
 template <bool IND>
-static cudaError_t launch_modes_wide_planes(const SweepParams& p, int lam, cudaStream_t s) {
-    if (p.accepts) return cudaErrorNotSupported;
-    if (p.G == 16) return launch_g_hm<16, IND>(p, lam, s);
-    return p.C % 32 == 0 ? launch_g_hm<32, IND>(p, lam, s) : cudaErrorNotSupported;
+static cudaError_t launch_modes_32(const SweepParams& p, int lam, cudaStream_t s) {
+    return p.accepts || p.C % 32 ? cudaErrorNotSupported : launch_g_hm<32, IND>(p, lam, s);
+}
+
+template <bool IND>
+static cudaError_t launch_modes_16(const SweepParams& p, int lam, cudaStream_t s) {
+    return p.accepts ? cudaErrorNotSupported : launch_g_hm<16, IND>(p, lam, s);
 }
 
 template <bool IND>

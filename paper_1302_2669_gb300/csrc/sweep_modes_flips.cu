@@ -4,7 +4,8 @@
 namespace surfmcmc {
 
 cudaError_t launch_sweep_modes_flips(const SweepParams& p, int lam, cudaStream_t s) {
-    return p.G >= 16 ? launch_modes_wide_planes<true>(p, lam, s) : cudaErrorNotSupported;
+    if (p.G == 16) return launch_modes_16<true>(p, lam, s);
+    return p.G == 32 ? launch_modes_32<true>(p, lam, s) : cudaErrorNotSupported;
 }
 
 }  // namespace surfmcmc

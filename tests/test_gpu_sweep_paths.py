@@ -29,9 +29,11 @@ def ctx(pkg):
     c.close()
 
 
-# error rates and beta* scales of the three compiled digit patterns: the first
-# eight binary digits of T[1..4] as (none, T1), (T1, T1 and T2), (any, any)
-TEMPS = {0: [(0.13, 1.0), (0.17, 1.0), (0.13, 0.4)], 1: [(0.05, 1.0), (0.08, 1.0), (0.05, 0.4)]}
+# error rates and beta* scales of the four compiled digit patterns: the first
+# eight binary digits of T[1..4] as (none, T1), (T1, T1 and T2), (any, any),
+# (T1, any)
+TEMPS = {0: [(0.13, 1.0), (0.17, 1.0), (0.13, 0.4), (0.13, 0.5)],
+         1: [(0.05, 1.0), (0.08, 1.0), (0.05, 0.4), (0.05, 0.5)]}
 
 
 # R: planes of 4, 8, 16 and 32 chains, the last also partly filled (9); n
