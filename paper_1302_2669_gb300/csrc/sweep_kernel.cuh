@@ -643,12 +643,13 @@ struct StartState {
 // 16-chain planes at 4 lanes; with 16-chain planes otherwise it costs 1 to 8
 // %, with 4-chain planes (eight ids) up to 2 %.  Counting accepts on 32-chain
 // planes takes 15 % longer without it (L = 25, 912 syndromes of 32 chains, 60
-// sweeps: 5.21 ms against 3.91).
+// sweeps: 5.21 ms against 3.91).  Full batches of 32-chain planes at 16 lanes
+// drop it as well (few_units).
 __host__ __device__ constexpr bool keep_map(int G, int lam) {
     return G == 8 || (G == 32 && lam != 4) || (G == 16 && lam == 4);
 }
 
-template <int G, int LAM, bool IND, bool ACPT, int HM>
+template <int G, int LAM, bool IND, bool ACPT, int HM, bool KEEP>
 __device__ __forceinline__ void run_unit(const SweepParams& p, const GroupDesc& gd, long long unit,
                                          uint32_t* smem, const ushort4* tab) {
     constexpr int B = 32 / LAM;                       // bundles per warp
@@ -675,7 +676,6 @@ __device__ __forceinline__ void run_unit(const SweepParams& p, const GroupDesc& 
     uint32_t* cfg = p.chain_frames ? p.chain_frames + gd.frames_off - (size_t)gd.item_base * p.C * 2 * W : nullptr;
     const BundleMap<G> bm(p, gd, bid);
     const uint32_t valid = bm.valid;
-    constexpr bool KEEP = keep_map(G, LAM);
     {
         if (sub == 0) {
             binfo[slot * (kMaxSlots + 1)] = bm.w;
@@ -874,7 +874,7 @@ __device__ __forceinline__ void run_unit(const SweepParams& p, const GroupDesc& 
 // fill its warps) first by its index, then from a queue counter, in the order
 // the host arranged (largest work first), and rebuilds the support table in
 // shared memory when the group's code size changes.
-template <int G, int LAM, bool IND, bool ACPT, int HM = 0>
+template <int G, int LAM, bool IND, bool ACPT, int HM = 0, bool KEEP = keep_map(G, LAM)>
 __global__ void __launch_bounds__(128, sweep_blocks_per_sm(G, LAM)) sweep_kernel(const __grid_constant__ SweepParams p) {
     extern __shared__ __align__(16) uint32_t smem[];
     __shared__ long long s_unit;
@@ -908,7 +908,7 @@ __global__ void __launch_bounds__(128, sweep_blocks_per_sm(G, LAM)) sweep_kernel
             cur = g;
             __syncthreads();
         }
-        run_unit<G, LAM, IND, ACPT, HM>(p, gd, u - gd.unit_base, smem, tab);
+        run_unit<G, LAM, IND, ACPT, HM, KEEP>(p, gd, u - gd.unit_base, smem, tab);
         __syncthreads();
         if (!p.unit_counter) break;
     }
@@ -938,14 +938,14 @@ struct SmemLimit {
     }
 };
 
-template <int G, int LAM, bool IND, bool ACPT = false, int HM = 0>
+template <int G, int LAM, bool IND, bool ACPT = false, int HM = 0, bool KEEP = keep_map(G, LAM)>
 static cudaError_t launch_t(const SweepParams& p, cudaStream_t s) {
     const size_t smem = sweep_smem_bytes(p.grp_nq_max, p.grp_nc_max, LAM) +
                         (ACPT ? (size_t)kWarps * kAcptWordsPerWarp * 4 : 0);
     static SmemLimit limit;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = limit.ensure(sweep_kernel<G, LAM, IND, ACPT, HM>, dev, smem);
+    if (e == cudaSuccess) e = limit.ensure(sweep_kernel<G, LAM, IND, ACPT, HM, KEEP>, dev, smem);
     if (e != cudaSuccess) return e;
     if (p.total_units == 0) return cudaSuccess;
     long long blocks = p.total_units;
@@ -954,7 +954,7 @@ static cudaError_t launch_t(const SweepParams& p, cudaStream_t s) {
         int sms = 0, per_sm = 0;
         e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (e == cudaSuccess)
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sweep_kernel<G, LAM, IND, ACPT, HM>, 32 * kWarps,
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sweep_kernel<G, LAM, IND, ACPT, HM, KEEP>, 32 * kWarps,
                                                               smem);
         if (e != cudaSuccess) return e;
         int bps = per_sm > 0 ? per_sm : 1;
@@ -964,7 +964,7 @@ static cudaError_t launch_t(const SweepParams& p, cudaStream_t s) {
         e = cudaMemsetAsync(p.unit_counter, 0, sizeof(unsigned int), s);
         if (e != cudaSuccess) return e;
     }
-    sweep_kernel<G, LAM, IND, ACPT, HM><<<(unsigned)blocks, 32 * kWarps, smem, s>>>(p);
+    sweep_kernel<G, LAM, IND, ACPT, HM, KEEP><<<(unsigned)blocks, 32 * kWarps, smem, s>>>(p);
     return cudaGetLastError();
 }
 

@@ -8,13 +8,31 @@
 
 namespace surfmcmc {
 
+// Whether a launch of 32-chain planes at 16 lanes fills less than half of the
+// device's resident blocks.  Such a launch runs at the latency of its units,
+// which is 2 to 6 % shorter with the bundle's map kept (L = 4 .. 13); fuller
+// ones run faster without it (16,384 syndromes of 64 chains at L = 13, 1,000
+// sweeps: 113.1 against 115.0 ms; at L = 17, 300 sweeps: 60.3 against 61.9) but
+// for some sizes with a short last wave (10,000 syndromes at L = 13, 600 sweeps:
+// 45.8 against 44.2).
+static inline bool few_units(const SweepParams& p) {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return true;
+    return 2 * p.total_units < (long long)sms * sweep_blocks_per_sm(32, 16);
+}
+
 template <int G, bool IND, int HM>
 static cudaError_t launch_hm(const SweepParams& p, int lam, cudaStream_t s) {
     switch (lam) {
         case 2: return launch_t<G, 2, IND, false, HM>(p, s);
         case 4: return launch_t<G, 4, IND, false, HM>(p, s);
         case 8: return launch_t<G, 8, IND, false, HM>(p, s);
-        case 16: return launch_t<G, 16, IND, false, HM>(p, s);
+        case 16:
+            if constexpr (G == 32)
+                if (!few_units(p)) return launch_t<G, 16, IND, false, HM, false>(p, s);
+            return launch_t<G, 16, IND, false, HM>(p, s);
         case 32: return launch_t<G, 32, IND, false, HM>(p, s);
         default: return cudaErrorNotSupported;
     }
