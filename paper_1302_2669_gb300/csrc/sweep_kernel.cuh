@@ -1,7 +1,8 @@
 // The Metropolis sweep kernel (Sec. IV / IV.A, parallelised as in Sec. V),
-// templated on the chain layout, the lanes per bundle and the noise model;
-// sweep.cu and sweep_flips.cu instantiate it for depolarizing
-// noise and for independent bit and phase flips.
+// templated on the chain layout, the lanes per bundle, the noise model and the
+// digit pattern; instantiated in sweep.cu and sweep_flips.cu (patterns read
+// from the parameters; depolarizing noise, independent flips) and in
+// sweep_modes*.cu (patterns compiled in).
 //
 // Data layout.  Chains are bit-sliced: a "bundle" holds 32 chains, and each
 // data qubit of a bundle is two 32-bit words in shared memory, X[q] and Z[q],
